@@ -142,15 +142,26 @@ int profile_restart(rng_gen *g, rng_err **err) {
   return rngi::cuda_fail(err, cudaEventRecord(g->origin, g->compute), "cudaEventRecord");
 }
 
+// Device memory of a launch whose tiles are split by rows (the jump table and,
+// with `second_state`, the second state array); false if it cannot be had.
+bool band_memory(rng_gen *g, bool second_state) {
+  if (second_state && !g->d_state2 && cudaMalloc(&g->d_state2, g->n * 8) != cudaSuccess) g->d_state2 = nullptr;
+  if (!g->d_jump && cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * 64 * 8) != cudaSuccess) g->d_jump = nullptr;
+  const bool ok = g->d_jump && (!second_state || g->d_state2);
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 // Prepares a banded launch of `a` with `br` rows per band: the second state
 // array (final states go there; the generator switches to it after the
 // launch) and the GF(2) jump table on the device.
-int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool *swap, rng_err **err) {
+// second_state: the launch's blocks read starting states that others replace.
+int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state, bool *swap, rng_err **err) {
   const uint64_t bands = (a.rows + br - 1) / br;
   if (bands > rngi::kMaxBands) return rngi::fail(err, RNG_EINVAL, "banded launch: %llu bands", (unsigned long long)bands);
   const uint32_t count = static_cast<uint32_t>(bands);  // one matrix per band
   int rc = RNG_OK;
-  if (!g->d_state2)
+  if (second_state && !g->d_state2)
     rc = rngi::cuda_fail(err, cudaMalloc(&g->d_state2, g->n * 8), "cudaMalloc(second state array)");
   if (!rc && !g->d_jump)
     rc = rngi::cuda_fail(err, cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * 64 * 8), "cudaMalloc(jump table)");
@@ -168,7 +179,7 @@ int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool *swap, rng_er
   }
   a.band_rows = br;
   a.jump = g->d_jump;
-  if (a.write_state) {
+  if (a.write_state && second_state) {
     a.state_out = g->d_state2;
     *swap = true;
   }
@@ -198,7 +209,7 @@ int gen_launch_rows(rng_gen *g, rngi::RowsLaunch &a, const rngi::LaunchShape &sh
   if (!a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n) {
     const uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
     if (br) {
-      int rc = setup_bands(g, a, br, &swap, err);
+      int rc = setup_bands(g, a, br, true, &swap, err);
       if (rc) return rc;
     }
   }
@@ -961,9 +972,8 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   if (iterations == 0) return RNG_OK;
   rc = size_ok(g->n, iterations, err);
   if (rc) return rc;
-  cudaError_t st = cudaMemsetAsync(row_xor_dev, 0, iterations * 8, g->compute);
-  if (st == cudaSuccess) st = cudaMemsetAsync(row_sum_dev, 0, iterations * 8, g->compute);
-  rc = rngi::cuda_fail(err, st, "cudaMemsetAsync(checksums)");
+  cudaError_t st = rngi::launch_zero_pair(row_xor_dev, row_sum_dev, iterations, g->compute);
+  rc = rngi::cuda_fail(err, st, "checksum reset launch");
   if (rc) return rc;
   rngi::RowsLaunch a{};
   a.state = g->d_state;
@@ -977,22 +987,46 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   a.from_hash = !g->materialized;
   a.write_state = 1;
   a.state_out = a.state;
-  const uint32_t v = g->opts.values_per_thread;
-  const uint32_t vpt = rngi::checksum_vpt(g->n, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0, g->device,
-                                           g->opts.output_mode);
-  // Few tiles, many rows: bands, as for the row kernel.
-  rngi::LaunchShape sh{};
-  sh.vpt = vpt;
-  sh.block = rngi::kGenBlock;
-  bool swap = false;
   a.out_mode = g->opts.output_mode;
-  const uint64_t br = rngi::choose_band_rows(g->n, iterations, sh, g->device, true, a.out_mode);
-  if (br) {
-    rc = setup_bands(g, a, br, &swap, err);
-    if (rc) return rc;
+  bool swap = false;
+  long op = -1;
+  // Launches that fill the GPU are split by rows except where a capture would
+  // record the jump table's upload from this call's memory, or one of two
+  // state arrays.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(g->compute, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  rngi::SlicedPlan plan;
+  if (!g->opts.values_per_thread && a.out_mode == 0) {
+    plan = rngi::choose_sliced(g->n, iterations, g->device, !capturing);
+    if (plan.quantum_rows && !band_memory(g, !a.from_hash))
+      plan = rngi::choose_sliced(g->n, iterations, g->device, false);
   }
-  long op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
-  st = rngi::launch_checksum(a, vpt, row_xor_dev, row_sum_dev, g->compute);
+  if (plan.blocks) {
+    if (plan.quantum_rows) {
+      rc = setup_bands(g, a, plan.quantum_rows, !a.from_hash, &swap, err);
+      if (rc) return rc;
+    }
+    op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
+    st = rngi::launch_checksum_sliced(a, plan, row_xor_dev, row_sum_dev, g->compute);
+  } else {
+    const uint32_t v = g->opts.values_per_thread;
+    const uint32_t vpt = rngi::checksum_vpt(g->n, iterations, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0);
+    // Few tiles, many rows: bands, as for the row kernel.
+    rngi::LaunchShape sh{};
+    sh.vpt = vpt;
+    sh.block = rngi::kGenBlock;
+    uint64_t br = rngi::choose_band_rows(g->n, iterations, sh, g->device, true, a.out_mode);
+    if (!br && !capturing) {
+      br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
+      if (br && !band_memory(g, !a.from_hash)) br = 0;
+    }
+    if (br) {
+      rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
+      if (rc) return rc;
+    }
+    op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
+    st = rngi::launch_checksum(a, vpt, row_xor_dev, row_sum_dev, g->compute);
+  }
   op_end(g, op, g->compute);
   rc = rngi::cuda_fail(err, st, "checksum kernel launch");
   if (rc) return rc;

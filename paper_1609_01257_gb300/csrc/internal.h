@@ -33,6 +33,11 @@ const void *rows_staged_kernel_fn(uint32_t vpt, bool banded, uint32_t out);
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out);
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb);
 const void *checksum_kernel_fn(uint32_t vpt, bool banded = false, uint32_t out = 0);
+// Bit-sliced generate-and-checksum kernel (output mode 0; checksum_sliced.cu):
+// blocks of kSlicedBlock threads, tiles of kSlicedTile streams.
+constexpr uint32_t kSlicedBlock = 128;
+constexpr uint64_t kSlicedTile = uint64_t(kSlicedBlock) * 64;
+const void *checksum_sliced_kernel_fn();
 const void *worklist_kernel_fn(uint32_t vpt);
 const void *batch_work_kernel_fn(uint32_t vpt);
 // Batched form with bulk copies for units of at least 16 rows: (4, 8),
@@ -42,6 +47,7 @@ const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb);
 const void *init_kernel_fn();
 const void *jump_kernel_fn();
 const void *copy_kernel_fn();
+const void *zero_pair_kernel_fn();
 
 // Sets *err (when err != NULL and *err == NULL) and returns `code`.
 int fail(rng_err **err, int code, const char *fmt, ...) __attribute__((format(printf, 3, 4)));
@@ -128,13 +134,28 @@ void jump_matrix(uint64_t k, uint64_t *cols);
 // of stream s (from the hash when from_hash).
 cudaError_t launch_jump(uint64_t *state, uint64_t n, uint64_t id_base, uint32_t key, int from_hash,
                         const uint64_t *cols, cudaStream_t st);
-// Values per thread of a generate-and-checksum launch over `span` streams
-// (vpt = 0: choose; else a power of two up to 64).
-uint32_t checksum_vpt(uint64_t span, uint32_t vpt, int device, uint32_t out_mode);
+// Values per thread of a generate-and-checksum launch of `rows` rows over
+// `span` streams (vpt = 0: choose; else a power of two up to 64).
+uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt);
+// x[0 .. n-1] = s[0 .. n-1] = 0 in one launch.
+cudaError_t launch_zero_pair(uint64_t *x, uint64_t *s, uint64_t n, cudaStream_t st);
 // Generate-and-checksum launch with `vpt` values per thread; a.band_rows != 0
 // selects the banded variant (a.jump, a.state_out as for the row kernel).
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,
                             cudaStream_t st);
+// How a generate-and-checksum launch runs bit-sliced: `blocks` blocks over
+// equal runs of (tile, quantum of `quantum_rows` rows) pairs; quantum_rows ==
+// 0: whole tiles; blocks == 0: the launch keeps checksum_kernel.
+struct SlicedPlan {
+  uint32_t blocks = 0;
+  uint64_t quantum_rows = 0;
+};
+// may_split: whether tiles may be split by rows (needs a.jump, and another
+// state_out when the states are in memory).
+SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_split);
+// a.band_rows = the plan's quantum_rows.
+cudaError_t launch_checksum_sliced(const RowsLaunch &a, const SlicedPlan &plan, uint64_t *row_xor, uint64_t *row_sum,
+                                   cudaStream_t st);
 int device_sm_count(int device);
 
 // Work-list kernel tables (batched and served forms).  One entry is a chunk
@@ -187,6 +208,10 @@ int batch_blocks_per_sm(uint32_t vpt, uint32_t block);
 // `checksum`: for the generate-and-checksum kernel instead of the row kernel.
 uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh, int device,
                           bool checksum = false, uint32_t out = 0);
+// Rows per band when a generate-and-checksum launch of more tiles than block
+// slots would leave its last wave mostly empty (1.7 waves of tiles cost two);
+// 0 for no split.
+uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int device, uint32_t out);
 // Most bands one banded launch is split into (one jump matrix each).
 constexpr uint32_t kMaxBands = 1024;
 // Host-side GF(2) tables for banded launches: writes `count` matrices

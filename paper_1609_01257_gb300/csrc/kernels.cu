@@ -20,6 +20,7 @@
 
 #include "internal.h"
 #include "prng_math.cuh"
+#include "reduce_jump.cuh"
 
 namespace rngi {
 namespace {
@@ -271,29 +272,6 @@ __device__ __forceinline__ bool rows_line_aligned(const uint64_t *row0, uint64_t
   return (reinterpret_cast<uintptr_t>(row0) & 127) == 0 && (pitch & 15) == 0;
 }
 
-// Nibble tables of a 64x64 matrix over GF(2) given by its columns (col[j] =
-// image of bit j): tab[q][e] = XOR of columns 4q+i over the bits i set in the
-// 4-bit value e.  The product with a vector is then 16 table reads and XORs
-// instead of 64 masked XORs, and each table is 16 words (128 bytes), so a
-// warp's reads of one table never conflict on the shared-memory banks.
-// Filled by the whole block.
-__device__ __forceinline__ void fill_jump_tables(uint64_t (*tab)[16], const uint64_t *__restrict__ cols) {
-  for (int idx = threadIdx.x; idx < 16 * 16; idx += blockDim.x) {
-    const int q = idx >> 4, e = idx & 15;
-    uint64_t acc = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc ^= cols[4 * q + i] & (0ull - static_cast<uint64_t>((e >> i) & 1));
-    tab[q][e] = acc;
-  }
-}
-
-__device__ __forceinline__ uint64_t apply_jump_tables(const uint64_t (*tab)[16], uint64_t x) {
-  uint64_t acc = 0;
-#pragma unroll
-  for (int q = 0; q < 16; ++q) acc ^= tab[q][(x >> (4 * q)) & 15];
-  return acc;
-}
-
 // Advances the states by band * band_rows iterations: one multiplication over
 // GF(2) by M^(band * band_rows), whose 64 columns are jump[64 band ..
 // 64 band + 63].  Called by every thread of the block (it synchronises the
@@ -432,6 +410,15 @@ __global__ void init_kernel(uint64_t *__restrict__ state, uint64_t n, uint64_t i
     state[s] = prng::initial_state(id_base + s, key);
 }
 
+// Clears two arrays of n words.
+__global__ void zero_pair_kernel(uint64_t *x, uint64_t *s, uint64_t n) {
+  for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < n;
+       i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+    x[i] = 0;
+    s[i] = 0;
+  }
+}
+
 // Jump-ahead: every state is multiplied by a 64x64 matrix over GF(2) given
 // by its columns (col[j] = image of bit j), i.e. advanced by the number of
 // iterations the matrix stands for.  The update is linear over GF(2), so k
@@ -472,37 +459,35 @@ __global__ void copy_kernel(uint64_t *__restrict__ dst, const uint64_t *__restri
   for (; i < n; i += stride) store_one<kPolicyStreaming>(dst + i, __ldcs(src + i));
 }
 
-// 64-bit XOR and wrapping sum across a warp with 32-bit reductions: the sum
-// is split into two 16-bit low parts (no carry can be lost over 32 lanes)
-// and the high word, whose sum only matters modulo 2^32.
-__device__ __forceinline__ void warp_xor_sum(uint64_t &x, uint64_t &s) {
-  const unsigned full = 0xffffffffu;
-  const uint32_t xl = __reduce_xor_sync(full, static_cast<uint32_t>(x));
-  const uint32_t xh = __reduce_xor_sync(full, static_cast<uint32_t>(x >> 32));
-  const uint32_t lo = static_cast<uint32_t>(s);
-  const uint32_t a = __reduce_add_sync(full, lo & 0xffffu);
-  const uint32_t b = __reduce_add_sync(full, lo >> 16);
-  const uint32_t c = __reduce_add_sync(full, static_cast<uint32_t>(s >> 32));
-  x = (static_cast<uint64_t>(xh) << 32) | xl;
-  s = static_cast<uint64_t>(a) + (static_cast<uint64_t>(b) << 16) + (static_cast<uint64_t>(c) << 32);
-}
-
 // Generate-and-checksum: per row, XOR and sum of all values of the launch's
-// stream range, reduced per warp, then per block (double-buffered shared
-// slots, one barrier per row), then one atomic pair per block and row.
+// stream range.  Bound by the ALU pipe (the update's shifts and XORs), so
+// everything else is kept off the row loop: each thread leaves its partial
+// sum of a row in shared memory, and every kChecksumRows rows one warp per
+// row adds the block's partials and does the row's atomics.  (A reduction by
+// `redux` in every warp and row, with one barrier a row, cost a fifth of all
+// instructions: 2^22 streams x 1024 rows 2508 us, now 2049 us, and 2629 us
+// for OUT = 1, 2882 before.)  Large OUT = 0 launches run bit-sliced instead
+// (checksum_sliced.cu).
+// OUT = 0: the update is linear over GF(2), so the XOR of a tile's values in
+// the next row is the update of their XOR in this one; it is reduced once per
+// unit and then stepped by one thread.  OUT = 1: the sum of the emitted
+// values is the multiplier times the sum of the states (modulo 2^64); the XOR
+// is taken over the emitted values.
 // Banded (BANDED = true): work units are (tile, band of band_rows rows), each
 // unit jumping its states ahead to its band over GF(2) as in the row kernel;
 // final states go to state_out (from the last band).
+constexpr int kChecksumRows = kBlock / 32;  // one warp per row of a batch
+
 template <int VPT, bool BANDED, int OUT = 0>
 __global__ void __launch_bounds__(kBlock) checksum_kernel(const RowsLaunch a,
                                                        unsigned long long *row_xor,
                                                        unsigned long long *row_sum) {
-  __shared__ uint64_t sx[2][kBlock / 32], ss[2][kBlock / 32];
+  __shared__ uint64_t part_s[kChecksumRows][kBlock];
+  __shared__ uint64_t part_x[OUT ? kChecksumRows : 1][kBlock];
   const uint64_t span = a.s_end - a.s_begin;
   const uint64_t tile_vals = static_cast<uint64_t>(kBlock) * VPT;
   const uint64_t n_tiles = (span + tile_vals - 1) / tile_vals;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int n_warps = kBlock / 32;
   const uint64_t band_rows = BANDED ? a.band_rows : (a.rows ? a.rows : 1);
   const uint64_t n_bands = BANDED ? (a.rows + band_rows - 1) / band_rows : 1;
   for (uint64_t w = blockIdx.x; w < n_tiles * n_bands; w += gridDim.x) {
@@ -515,39 +500,53 @@ __global__ void __launch_bounds__(kBlock) checksum_kernel(const RowsLaunch a,
       __shared__ uint64_t jtab[16][16];
       if (band) jump_states<VPT>(st, a.jump, band, jtab);  // band is the same for the whole block
     }
+    // Values past the end of the range were loaded as 0 and advance to 0, so
+    // they add nothing to either checksum.
+    uint64_t tile_xor = 0;
+    if constexpr (OUT == 0) {
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) tile_xor ^= st[v];
+      tile_xor = block_xor<kBlock>(tile_xor, &part_x[0][0]);
+    }
     const uint64_t r0 = band * band_rows;
     const uint64_t rows = BANDED ? (a.rows - r0 < band_rows ? a.rows - r0 : band_rows) : a.rows;
-    for (uint64_t r = 0; r < rows; ++r) {
-      uint64_t x = 0, s = 0;
+    for (uint64_t r = 0; r < rows; r += kChecksumRows) {
+      const int m = rows - r < kChecksumRows ? static_cast<int>(rows - r) : kChecksumRows;
+#pragma unroll 1
+      for (int q = 0; q < m; ++q) {
+        uint64_t x = 0, s = 0;
 #pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        const uint64_t e = prng::emitted<OUT>(st[v]);
-        x ^= e;
-        s += e;
-        st[v] = prng::xorshift_update(st[v]);
-      }
-      warp_xor_sum(x, s);
-      const int buf = static_cast<int>(r & 1);
-      if (lane == 0) {
-        sx[buf][warp] = x;
-        ss[buf][warp] = s;
+        for (int v = 0; v < VPT; ++v) {
+          s += st[v];
+          if constexpr (OUT != 0) x ^= prng::emitted<OUT>(st[v]);
+          st[v] = prng::xorshift_update(st[v]);
+        }
+        part_s[q][threadIdx.x] = s;
+        if constexpr (OUT != 0) part_x[q][threadIdx.x] = x;
       }
       __syncthreads();
-      if (warp == 0) {
-        uint64_t bx = lane < n_warps ? sx[buf][lane] : 0;
-        uint64_t bs = lane < n_warps ? ss[buf][lane] : 0;
-        warp_xor_sum(bx, bs);
+      if (warp < m) {
+        uint64_t x = 0, s = 0;
+#pragma unroll
+        for (int i = 0; i < kBlock / 32; ++i) {
+          s += part_s[warp][lane + 32 * i];
+          if constexpr (OUT != 0) x ^= part_x[warp][lane + 32 * i];
+        }
+        warp_xor_sum(x, s);
         if (lane == 0) {
-          atomicXor(row_xor + r0 + r, static_cast<unsigned long long>(bx));
-          atomicAdd(row_sum + r0 + r, static_cast<unsigned long long>(bs));
+          atomicAdd(row_sum + r0 + r + warp, static_cast<unsigned long long>(prng::emitted<OUT>(s)));
+          if constexpr (OUT != 0) atomicXor(row_xor + r0 + r + warp, static_cast<unsigned long long>(x));
         }
       }
+      if (OUT == 0 && threadIdx.x == 0)
+        for (int q = 0; q < m; ++q) {
+          atomicXor(row_xor + r0 + r + q, static_cast<unsigned long long>(tile_xor));
+          tile_xor = prng::xorshift_update(tile_xor);
+        }
+      __syncthreads();
     }
-    // Values past the end of the range were loaded as 0 and advance to 0,
-    // so they add nothing; the states of real streams are written back.
     if (a.write_state && band == n_bands - 1)
       store_tile_state<VPT, 1>(st, BANDED ? a.state_out : a.state, a, rel0, span);
-    __syncthreads();
   }
 }
 
@@ -962,6 +961,7 @@ const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb) {
 }
 const void *init_kernel_fn() { return reinterpret_cast<const void *>(&init_kernel); }
 const void *jump_kernel_fn() { return reinterpret_cast<const void *>(&jump_kernel); }
+const void *zero_pair_kernel_fn() { return reinterpret_cast<const void *>(&zero_pair_kernel); }
 const void *copy_kernel_fn() { return reinterpret_cast<const void *>(&copy_kernel); }
 
 }  // namespace rngi

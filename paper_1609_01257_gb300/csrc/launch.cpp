@@ -387,6 +387,26 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
   return (rows + bands - 1) / bands;
 }
 
+uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int device, uint32_t out) {
+  const uint64_t tile = uint64_t(kGenBlock) * vpt, tiles = (streams + tile - 1) / tile;
+  const void *fn = checksum_kernel_fn(vpt, true, out);
+  if (!fn) return 0;
+  const uint64_t slots = static_cast<uint64_t>(device_sm_count(device)) * occupancy(fn, kGenBlock);
+  const auto use = [&](uint64_t units) {
+    return static_cast<double>(units) / static_cast<double>((units + slots - 1) / slots * slots);
+  };
+  if (tiles < slots || use(tiles) > 0.93) return 0;
+  double best = use(tiles) + 0.02;
+  uint64_t band = 0;
+  for (uint64_t bands = 2; bands <= 8 && rows / bands >= 64; ++bands) {
+    const uint64_t br = (rows + bands - 1) / bands;
+    if (use(tiles * ((rows + br - 1) / br)) <= best) continue;
+    best = use(tiles * ((rows + br - 1) / br));
+    band = br;
+  }
+  return band;
+}
+
 void jump_matrix(uint64_t k, uint64_t *cols) {
   const Gf2 m = update_power(k);
   for (int j = 0; j < 64; ++j) cols[j] = m.col[j];
@@ -407,20 +427,32 @@ cudaError_t launch_jump(uint64_t *state, uint64_t n, uint64_t id_base, uint32_t 
   return e;
 }
 
-uint32_t checksum_vpt(uint64_t span, uint32_t vpt, int device, uint32_t out_mode) {
-  (void)device;
+uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
   if (vpt) return vpt;
-  // 16 values per thread amortise the per-row reductions best (2^22 and 2^26
-  // streams: 1.72e12 values/s at 16, 1.38e12 at 8); runs with few tiles are
-  // banded to fill the GPU (2^18 streams: 1.21e12 banded at 16 vs 0.83e12
-  // unbanded at 8).  Up to 2^18 streams (banded launches) 32 are faster
-  // still in output mode 0 (2^16 and 2^18 streams: 1.73e12 at 32, 1.64e12 at
-  // 16; from 2^20 streams 16 is best: 1.55e12 vs 1.47e12 at 32).  Smaller
-  // values only when one tile would be mostly empty.
-  if (out_mode == 0 && span <= (uint64_t(1) << 18) && span >= uint64_t(kGenBlock) * 32) return 32;
-  for (uint32_t v = 16; v >= 2; v /= 2)
-    if (span >= uint64_t(kGenBlock) * v) return v;
-  return 1;
+  // Large launches run at the ALU rate with 8 to 32 values per thread; the
+  // start of a unit (jump, reductions) weighs least at 16.  Small launches are
+  // bound by one block's rows, one after another, so they take fewer values
+  // per thread and more blocks (us on GB300 at 4 / 8 / 16: 8192 x 1024 25 / 30
+  // / 40; 65536 x 256 32 / 31 / 40; 1000003 x 16 37 / 27 / 29; 262144 x 256
+  // 62 / 62 / 60; 65536 x 4096 176 / 167 / 173).  A tile that would be mostly
+  // past the end of the streams is halved.
+  const uint64_t values = span * rows;
+  uint32_t v = values >= (uint64_t(1) << 26) ? 16 : values >= (uint64_t(1) << 24) ? 8 : 4;
+  while (v > 1) {
+    const uint64_t tile = uint64_t(kGenBlock) * v, tiles = (span + tile - 1) / tile;
+    if (span * 5 >= tiles * tile * 4) break;
+    if (tiles > 8) break;
+    v /= 2;
+  }
+  return v;
+}
+
+cudaError_t launch_zero_pair(uint64_t *x, uint64_t *s, uint64_t n, cudaStream_t st) {
+  const uint64_t blocks = std::min<uint64_t>((n + 255) / 256, 1024);
+  void *params[] = {&x, &s, &n};
+  const cudaError_t e = cudaLaunchKernel(zero_pair_kernel_fn(), dim3(static_cast<unsigned>(blocks)), dim3(256), params, 0, st);
+  if (e == cudaSuccess) count_launch();
+  return e;
 }
 
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,
@@ -429,7 +461,7 @@ cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor
   int dev = 0;
   cudaGetDevice(&dev);
   const int sms = device_sm_count(dev);
-  if (a.band_rows && (!a.jump || (a.write_state && a.state_out == a.state))) return cudaErrorInvalidValue;
+  if (a.band_rows && (!a.jump || (a.write_state && !a.from_hash && a.state_out == a.state))) return cudaErrorInvalidValue;
   const void *fn = checksum_kernel_fn(vpt, a.band_rows != 0, a.out_mode);
   if (!fn) return cudaErrorInvalidValue;
   const uint64_t tiles = (span + uint64_t(kGenBlock) * vpt - 1) / (uint64_t(kGenBlock) * vpt);
@@ -441,6 +473,54 @@ cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor
   unsigned long long *rs = reinterpret_cast<unsigned long long *>(row_sum);
   void *params[] = {&args, &rx, &rs};
   cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(kGenBlock), params, 0, st);
+  if (e == cudaSuccess) count_launch();
+  return e;
+}
+
+SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_split) {
+  SlicedPlan p;
+  const uint64_t tiles = (streams + kSlicedTile - 1) / kSlicedTile;
+  // A partly filled last tile costs as much as a full one.
+  if (streams * 3 < tiles * kSlicedTile * 2) return p;
+  // Each tile pays for its states' way into bit planes and back, and small
+  // launches need more blocks than there are tiles: us bit-sliced / best
+  // checksum_kernel shape on GB300: 2^24 x 64 450 / 519, 2^22 x 64 144 / 147,
+  // 2^20 x 128 88 / 96, 2^18 x 1024 130 / 166; below 2^27 values 2^18 x 256
+  // 64 / 60, 65536 x 1024 65 / 60, 2^18 x 128 56 / 40.
+  if (rows < 64 || streams * rows < (uint64_t(1) << 27)) return p;
+  const uint64_t slots = static_cast<uint64_t>(device_sm_count(device)) *
+                         static_cast<uint64_t>(occupancy(checksum_sliced_kernel_fn(), kSlicedBlock));
+  const uint64_t waves = (tiles + slots - 1) / slots;
+  const double whole = static_cast<double>(tiles) / static_cast<double>(waves * slots);  // share of the slots in use
+  p.blocks = static_cast<uint32_t>(std::min(tiles, uint64_t(0x7fffffff)));
+  if (!may_split || whole > 0.97) return p;
+  // The fewest quanta per tile (each is one matrix to compute and upload)
+  // that leave the longest run within 3 % of the mean; at least 16 rows each.
+  double best = whole;
+  for (uint64_t nq = 2; nq <= std::min<uint64_t>(rows / 16, kMaxBands); ++nq) {
+    const uint64_t q = (rows + nq - 1) / nq;
+    if ((rows + q - 1) / q != nq) continue;
+    const uint64_t blocks = std::min(slots, tiles * nq);
+    const uint64_t longest = (tiles * nq + blocks - 1) / blocks;
+    const double use = static_cast<double>(tiles) * static_cast<double>(rows) /
+                       (static_cast<double>(longest) * static_cast<double>(q) * static_cast<double>(slots));
+    if (use <= best) continue;
+    best = use;
+    p.blocks = static_cast<uint32_t>(blocks);
+    p.quantum_rows = q;
+    if (use > 0.97) break;
+  }
+  return p;
+}
+
+cudaError_t launch_checksum_sliced(const RowsLaunch &a, const SlicedPlan &plan, uint64_t *row_xor, uint64_t *row_sum,
+                                   cudaStream_t st) {
+  if (!plan.blocks || (a.band_rows && !a.jump)) return cudaErrorInvalidValue;
+  RowsLaunch args = a;
+  unsigned long long *rx = reinterpret_cast<unsigned long long *>(row_xor);
+  unsigned long long *rs = reinterpret_cast<unsigned long long *>(row_sum);
+  void *params[] = {&args, &rx, &rs};
+  cudaError_t e = cudaLaunchKernel(checksum_sliced_kernel_fn(), dim3(plan.blocks), dim3(kSlicedBlock), params, 0, st);
   if (e == cudaSuccess) count_launch();
   return e;
 }
