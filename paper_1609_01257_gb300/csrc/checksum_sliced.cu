@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kBlock, 3) checksum_sliced_kernel(const RowsLa
     const uint64_t r1 = q1 * quantum < a.rows ? q1 * quantum : a.rows;
     const uint64_t rel0 = tile * kSlicedTile + threadIdx.x;
     if (q0) {
-      fill_jump_tables(jtab, a.jump + 64 * q0);
+      load_jump_tables(jtab, a.jump + kJumpTableWords * q0);
       __syncthreads();
     }
     // One group at a time: the thread's 32 states go to its own column of

@@ -61,9 +61,9 @@ struct rng_gen {
   uint64_t chunk_span = 0;
   uint64_t *d_state = nullptr;
   uint64_t *d_state2 = nullptr;      // second state array for banded launches
-  uint64_t *d_jump = nullptr;        // GF(2) jump matrices for banded launches
+  uint64_t *d_jump = nullptr;        // GF(2) jump tables for banded launches
   uint64_t jump_rows = 0;            // band_rows the table on the device is for
-  uint32_t jump_count = 0;           // matrices in that table
+  uint32_t jump_count = 0;           // bands in that table
   cudaStream_t compute = nullptr, copy = nullptr;
   bool own_compute = false;
   uint64_t *d_buf[2] = {nullptr, nullptr};
@@ -146,7 +146,7 @@ int profile_restart(rng_gen *g, rng_err **err) {
 // with `second_state`, the second state array); false if it cannot be had.
 bool band_memory(rng_gen *g, bool second_state) {
   if (second_state && !g->d_state2 && cudaMalloc(&g->d_state2, g->n * 8) != cudaSuccess) g->d_state2 = nullptr;
-  if (!g->d_jump && cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * 64 * 8) != cudaSuccess) g->d_jump = nullptr;
+  if (!g->d_jump && cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * rngi::kJumpTableWords * 8) != cudaSuccess) g->d_jump = nullptr;
   const bool ok = g->d_jump && (!second_state || g->d_state2);
   if (!ok) cudaGetLastError();
   return ok;
@@ -164,15 +164,10 @@ int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state,
   if (second_state && !g->d_state2)
     rc = rngi::cuda_fail(err, cudaMalloc(&g->d_state2, g->n * 8), "cudaMalloc(second state array)");
   if (!rc && !g->d_jump)
-    rc = rngi::cuda_fail(err, cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * 64 * 8), "cudaMalloc(jump table)");
+    rc = rngi::cuda_fail(err, cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * rngi::kJumpTableWords * 8), "cudaMalloc(jump table)");
   if (rc) return rc;
   if (g->jump_rows != br || g->jump_count < count) {
-    std::vector<uint64_t> cols(size_t(count) * 64);
-    rngi::jump_table(br, count, cols.data());
-    // Pageable source: the call returns once the source has been read.
-    rc = rngi::cuda_fail(err, cudaMemcpyAsync(g->d_jump, cols.data(), cols.size() * 8, cudaMemcpyHostToDevice,
-                                              g->compute),
-                         "jump table upload");
+    rc = rngi::cuda_fail(err, rngi::launch_jump_tables(g->d_jump, br, count, g->compute), "jump table launch");
     if (rc) return rc;
     g->jump_rows = br;
     g->jump_count = count;
@@ -991,8 +986,7 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   bool swap = false;
   long op = -1;
   // Launches that fill the GPU are split by rows except where a capture would
-  // record the jump table's upload from this call's memory, or one of two
-  // state arrays.
+  // record one of two state arrays.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(g->compute, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
   rngi::SlicedPlan plan;

@@ -45,7 +45,6 @@ const void *batch_work_kernel_fn(uint32_t vpt);
 // rows_bulk_smem_bytes(vpt, nb).
 const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb);
 const void *init_kernel_fn();
-const void *jump_kernel_fn();
 const void *copy_kernel_fn();
 const void *zero_pair_kernel_fn();
 
@@ -74,7 +73,7 @@ struct RowsLaunch {
   int write_state;      // store the advanced states back
   uint64_t ring_rows;   // 0, or rows wrap around a ring of this many rows
   uint64_t band_rows;   // 0, or rows are split into bands of this many rows
-  const uint64_t *jump; // bands: matrices M^(band * band_rows) for band = 0, 1, ..., 64 columns each
+  const uint64_t *jump; // bands: nibble tables of M^(band * band_rows), band = 0, 1, ... (kJumpTableWords each)
   uint64_t *state_out;  // where final states go (== state unless banded)
   uint32_t out_mode;    // value emitted per state: 0 the state, 1 xorshift64* (selects the kernel)
 };
@@ -128,7 +127,16 @@ cudaError_t launch_init(uint64_t *state, uint64_t n, uint64_t id_base, uint32_t 
 // n words from device memory `src` to page-locked host memory `dst` (a
 // device-side address) by SMs, on stream st.
 cudaError_t launch_copy(uint64_t *dst, const uint64_t *src, uint64_t n, cudaStream_t st);
-// Columns of M^k, where M is the update's matrix over GF(2) (host side).
+// Jump-ahead (jump.cu).  Nibble tables of M^(band * band_rows), band = 0 ..
+// count - 1, M the update's matrix over GF(2), written to `tables` (device
+// memory, kJumpTableWords each) by one launch.
+constexpr uint32_t kJumpTableWords = 256;
+cudaError_t launch_jump_tables(uint64_t *tables, uint64_t band_rows, uint32_t count, cudaStream_t st);
+// From this many streams on rng_skip runs jump_wide_kernel (us per call in
+// series on GB300, jump_kernel / jump_wide_kernel: 2^20 8.3 / 10.3, 2^24 80 /
+// 56, 2^26 300 / 197; its tables cost about 4 us).
+constexpr uint64_t kJumpWideStreams = uint64_t(3) << 20;
+// Columns of M^k (host side).
 void jump_matrix(uint64_t k, uint64_t *cols);
 // state[s] := the matrix with columns `cols` (64 words) applied to the state
 // of stream s (from the hash when from_hash).
@@ -214,9 +222,6 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
 uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int device, uint32_t out);
 // Most bands one banded launch is split into (one jump matrix each).
 constexpr uint32_t kMaxBands = 1024;
-// Host-side GF(2) tables for banded launches: writes `count` matrices
-// M^(band * band_rows), band = 0 .. count-1, as 64 column words each.
-void jump_table(uint64_t band_rows, uint32_t count, uint64_t *cols);
 // Values per thread the work-list kernel is compiled for.
 bool batch_vpt_supported(uint32_t vpt);
 

@@ -11,8 +11,7 @@
 // and once at the end.
 //
 // Also here: the generate-and-checksum kernel, the work-list kernels of the
-// batched, served and allocation-free forms, the init and jump-ahead kernels,
-// and the copy kernel of the double buffer's copy-kernel reads.
+// batched, served and allocation-free forms, the init kernel, and the copy kernel of the double buffer's copy-kernel reads.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -273,14 +272,14 @@ __device__ __forceinline__ bool rows_line_aligned(const uint64_t *row0, uint64_t
 }
 
 // Advances the states by band * band_rows iterations: one multiplication over
-// GF(2) by M^(band * band_rows), whose 64 columns are jump[64 band ..
-// 64 band + 63].  Called by every thread of the block (it synchronises the
+// GF(2) by M^(band * band_rows), whose nibble tables are jump[256 band ..
+// 256 band + 255].  Called by every thread of the block (it synchronises the
 // block around refilling the shared tables).
 template <int VPT>
 __device__ __forceinline__ void jump_states(uint64_t (&st)[VPT], const uint64_t *__restrict__ jump,
                                             uint64_t band, uint64_t (*tab)[16]) {
   __syncthreads();  // the previous unit's reads of the tables are done
-  fill_jump_tables(tab, jump + 64 * band);
+  load_jump_tables(tab, jump + kJumpTableWords * band);
   __syncthreads();
 #pragma unroll
   for (int v = 0; v < VPT; ++v) st[v] = apply_jump_tables(tab, st[v]);
@@ -416,28 +415,6 @@ __global__ void zero_pair_kernel(uint64_t *x, uint64_t *s, uint64_t n) {
        i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     x[i] = 0;
     s[i] = 0;
-  }
-}
-
-// Jump-ahead: every state is multiplied by a 64x64 matrix over GF(2) given
-// by its columns (col[j] = image of bit j), i.e. advanced by the number of
-// iterations the matrix stands for.  The update is linear over GF(2), so k
-// iterations are the k-th power of its matrix.
-struct JumpMatrix {
-  uint64_t col[64];
-};
-
-// The product goes through the nibble tables above, which each block fills
-// from the matrix (a kernel parameter).
-__global__ void jump_kernel(uint64_t *__restrict__ state, uint64_t n, uint64_t id_base, uint32_t key,
-                            int from_hash, const __grid_constant__ JumpMatrix m) {
-  __shared__ uint64_t tab[16][16];
-  fill_jump_tables(tab, m.col);
-  __syncthreads();
-  for (uint64_t s = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; s < n;
-       s += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-    const uint64_t v = from_hash ? prng::initial_state(id_base + s, key) : state[s];
-    state[s] = apply_jump_tables(tab, v);
   }
 }
 
@@ -960,7 +937,6 @@ const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb) {
   return nullptr;
 }
 const void *init_kernel_fn() { return reinterpret_cast<const void *>(&init_kernel); }
-const void *jump_kernel_fn() { return reinterpret_cast<const void *>(&jump_kernel); }
 const void *zero_pair_kernel_fn() { return reinterpret_cast<const void *>(&zero_pair_kernel); }
 const void *copy_kernel_fn() { return reinterpret_cast<const void *>(&copy_kernel); }
 

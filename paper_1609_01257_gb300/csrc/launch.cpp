@@ -1,6 +1,6 @@
 // Host-side launch code of the kernels: shape selection (values per thread,
-// store width, grid, bands), the GF(2) jump matrices of rng_skip and of
-// banded launches, and the launches themselves.  The kernels are in
+// store width, grid, bands) and the launches themselves, but for the
+// jump-ahead's (jump.cu).  The kernels are in
 // kernels.cu; this file holds no device code.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -290,69 +290,6 @@ cudaError_t launch_copy(uint64_t *dst, const uint64_t *src, uint64_t n, cudaStre
   return e;
 }
 
-namespace {
-
-// 64x64 matrices over GF(2) as 64 column words (column j = image of bit j).
-struct Gf2 {
-  uint64_t col[64];
-};
-
-// a * b over GF(2) (apply b first).  Each column of b is multiplied through
-// byte tables of a: tab[q][e] = XOR of a's columns 8q+i over the bits i of
-// e, each entry one XOR from a smaller one, then 8 lookups per column.
-Gf2 gf2_mul(const Gf2 &a, const Gf2 &b) {
-  static thread_local uint64_t tab[8][256];
-  for (int q = 0; q < 8; ++q) {
-    tab[q][0] = 0;
-    for (int e = 1; e < 256; ++e) tab[q][e] = tab[q][e & (e - 1)] ^ a.col[8 * q + __builtin_ctz(e)];
-  }
-  Gf2 r;
-  for (int j = 0; j < 64; ++j) {
-    uint64_t acc = 0;
-    for (int q = 0; q < 8; ++q) acc ^= tab[q][(b.col[j] >> (8 * q)) & 255];
-    r.col[j] = acc;
-  }
-  return r;
-}
-
-Gf2 gf2_identity() {
-  Gf2 r;
-  for (int j = 0; j < 64; ++j) r.col[j] = uint64_t(1) << j;
-  return r;
-}
-
-// M^(2^i), i = 0 .. 63, for the xorshift update M (columns of M are the
-// update of each unit vector), built once by repeated squaring.
-const Gf2 *update_powers_of_two() {
-  static const std::vector<Gf2> pw = [] {
-    std::vector<Gf2> v(64);
-    for (int j = 0; j < 64; ++j) v[0].col[j] = prng::xorshift_update(uint64_t(1) << j);
-    for (int i = 1; i < 64; ++i) v[i] = gf2_mul(v[i - 1], v[i - 1]);
-    return v;
-  }();
-  return pw.data();
-}
-
-// M^k: one product per set bit of k.
-Gf2 update_power(uint64_t k) {
-  const Gf2 *pw = update_powers_of_two();
-  Gf2 result = gf2_identity();
-  for (int i = 0; k; ++i, k >>= 1)
-    if (k & 1) result = gf2_mul(pw[i], result);
-  return result;
-}
-
-}  // namespace
-
-void jump_table(uint64_t band_rows, uint32_t count, uint64_t *cols) {
-  const Gf2 step = update_power(band_rows);
-  Gf2 m = gf2_identity();  // band 0 starts at the launch's first row
-  for (uint32_t b = 0; b < count; ++b) {
-    for (int j = 0; j < 64; ++j) cols[64 * b + j] = m.col[j];
-    m = gf2_mul(step, m);
-  }
-}
-
 // Row kernel (bound by HBM writes): bands only when the tiles cannot cover
 // half the SMs (128 unbanded tiles of 2^16 streams ran at 7.37 TB/s, three
 // bands of them at 6.25); then about two (tile, band) units per SM (16 tiles
@@ -365,7 +302,7 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
                           uint32_t out) {
   const uint64_t sms = static_cast<uint64_t>(device_sm_count(device));
   const uint64_t tiles = (streams + uint64_t(sh.block) * sh.vpt - 1) / (uint64_t(sh.block) * sh.vpt);
-  const uint64_t min_band = 128;
+  const uint64_t min_band = checksum ? 64 : 128;
   const void *fn = checksum     ? checksum_kernel_fn(sh.vpt, true, out)
                    : sh.bulk_nb ? rows_bulk_kernel_fn(sh.vpt, sh.bulk_nb, true, out)
                    : sh.staged  ? rows_staged_kernel_fn(sh.vpt, true, out)
@@ -405,26 +342,6 @@ uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int 
     band = br;
   }
   return band;
-}
-
-void jump_matrix(uint64_t k, uint64_t *cols) {
-  const Gf2 m = update_power(k);
-  for (int j = 0; j < 64; ++j) cols[j] = m.col[j];
-}
-
-cudaError_t launch_jump(uint64_t *state, uint64_t n, uint64_t id_base, uint32_t key, int from_hash,
-                        const uint64_t *cols, cudaStream_t st) {
-  Gf2 m;
-  for (int j = 0; j < 64; ++j) m.col[j] = cols[j];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const uint64_t blocks_needed = (n + 255) / 256;
-  const uint64_t cap = static_cast<uint64_t>(device_sm_count(dev)) * 8;
-  const unsigned grid = static_cast<unsigned>(blocks_needed < cap ? blocks_needed : cap);
-  void *params[] = {&state, &n, &id_base, &key, &from_hash, &m};
-  cudaError_t e = cudaLaunchKernel(jump_kernel_fn(), dim3(grid ? grid : 1), dim3(256), params, 0, st);
-  if (e == cudaSuccess) count_launch();
-  return e;
 }
 
 uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {

@@ -5,12 +5,13 @@
 
 namespace rngi {
 
-// Nibble tables of a 64x64 matrix over GF(2) given by its columns (col[j] =
-// image of bit j): tab[q][e] = XOR of columns 4q+i over the bits i set in the
-// 4-bit value e.  The product with a vector is then 16 table reads and XORs
-// instead of 64 masked XORs, and each table is 16 words (128 bytes), so a
-// warp's reads of one table never conflict on the shared-memory banks.
-// Filled by the whole block.
+// Nibble tables of a 64x64 matrix over GF(2): tab[q][e] = the matrix applied
+// to the 4-bit value e at bits 4q .. 4q+3.  The product with a vector is then
+// 16 table reads and XORs instead of 64 masked XORs, and each table is 16
+// words (128 bytes), so a warp's reads of one table never conflict on the
+// shared-memory banks.
+
+// From the matrix's columns (col[j] = image of bit j).  By the whole block.
 __device__ __forceinline__ void fill_jump_tables(uint64_t (*tab)[16], const uint64_t *__restrict__ cols) {
   for (int idx = threadIdx.x; idx < 16 * 16; idx += blockDim.x) {
     const int q = idx >> 4, e = idx & 15;
@@ -19,6 +20,11 @@ __device__ __forceinline__ void fill_jump_tables(uint64_t (*tab)[16], const uint
     for (int i = 0; i < 4; ++i) acc ^= cols[4 * q + i] & (0ull - static_cast<uint64_t>((e >> i) & 1));
     tab[q][e] = acc;
   }
+}
+
+// From the tables in memory that jump_tables_kernel wrote.  By the whole block.
+__device__ __forceinline__ void load_jump_tables(uint64_t (*tab)[16], const uint64_t *__restrict__ from) {
+  for (int idx = threadIdx.x; idx < 16 * 16; idx += blockDim.x) (&tab[0][0])[idx] = from[idx];
 }
 
 __device__ __forceinline__ uint64_t apply_jump_tables(const uint64_t (*tab)[16], uint64_t x) {
