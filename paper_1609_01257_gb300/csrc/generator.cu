@@ -64,6 +64,8 @@ struct rng_gen {
   uint64_t *d_jump = nullptr;        // GF(2) jump tables for banded launches
   uint64_t jump_rows = 0;            // band_rows the table on the device is for
   uint32_t jump_count = 0;           // bands in that table
+  uint32_t jump_cap = 0;             // bands it has room for
+  uint64_t *d_jump_small = nullptr;  // the table before it grew
   cudaStream_t compute = nullptr, copy = nullptr;
   bool own_compute = false;
   uint64_t *d_buf[2] = {nullptr, nullptr};
@@ -142,29 +144,45 @@ int profile_restart(rng_gen *g, rng_err **err) {
   return rngi::cuda_fail(err, cudaEventRecord(g->origin, g->compute), "cudaEventRecord");
 }
 
-// Device memory of a launch whose tiles are split by rows (the jump table and,
-// with `second_state`, the second state array); false if it cannot be had.
-bool band_memory(rng_gen *g, bool second_state) {
-  if (second_state && !g->d_state2 && cudaMalloc(&g->d_state2, g->n * 8) != cudaSuccess) g->d_state2 = nullptr;
-  if (!g->d_jump && cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * rngi::kJumpTableWords * 8) != cudaSuccess) g->d_jump = nullptr;
-  const bool ok = g->d_jump && (!second_state || g->d_state2);
-  if (!ok) cudaGetLastError();
-  return ok;
+// Device memory of a launch in `bands` bands: the jump tables and, with
+// `second_state`, the second state array.  Sized for what is asked (a table
+// for every SM's band is 320 KB, which cudaMalloc gives in microseconds where
+// 2 MB take about 100), so a generator's first banded launch does not wait
+// for it.
+cudaError_t band_memory(rng_gen *g, uint32_t bands, bool second_state) {
+  if (second_state && !g->d_state2) {
+    const cudaError_t e = cudaMalloc(&g->d_state2, g->n * 8);
+    if (e != cudaSuccess) {
+      g->d_state2 = nullptr;
+      cudaGetLastError();
+      return e;
+    }
+  }
+  if (g->jump_cap < bands) {
+    const uint32_t cap = bands <= 160 ? 160 : rngi::kMaxBands;
+    uint64_t *p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, size_t(cap) * rngi::kJumpTableWords * 8);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
+    g->d_jump_small = g->d_jump;  // launches in flight may read it: freed with the generator
+    g->d_jump = p;
+    g->jump_cap = cap;
+    g->jump_rows = 0;
+  }
+  return cudaSuccess;
 }
 
-// Prepares a banded launch of `a` with `br` rows per band: the second state
-// array (final states go there; the generator switches to it after the
-// launch) and the GF(2) jump table on the device.
-// second_state: the launch's blocks read starting states that others replace.
+// Prepares a banded launch of `a` with `br` rows per band: the jump tables on
+// the device and, where blocks read starting states that others replace
+// (second_state), the second state array (final states go there; the
+// generator switches to it after the launch).
 int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state, bool *swap, rng_err **err) {
   const uint64_t bands = (a.rows + br - 1) / br;
   if (bands > rngi::kMaxBands) return rngi::fail(err, RNG_EINVAL, "banded launch: %llu bands", (unsigned long long)bands);
-  const uint32_t count = static_cast<uint32_t>(bands);  // one matrix per band
-  int rc = RNG_OK;
-  if (second_state && !g->d_state2)
-    rc = rngi::cuda_fail(err, cudaMalloc(&g->d_state2, g->n * 8), "cudaMalloc(second state array)");
-  if (!rc && !g->d_jump)
-    rc = rngi::cuda_fail(err, cudaMalloc(&g->d_jump, size_t(rngi::kMaxBands) * rngi::kJumpTableWords * 8), "cudaMalloc(jump table)");
+  const uint32_t count = static_cast<uint32_t>(bands);
+  int rc = rngi::cuda_fail(err, band_memory(g, count, second_state), "cudaMalloc(second state array, jump tables)");
   if (rc) return rc;
   if (g->jump_rows != br || g->jump_count < count) {
     rc = rngi::cuda_fail(err, rngi::launch_jump_tables(g->d_jump, br, count, g->compute), "jump table launch");
@@ -197,14 +215,19 @@ int gen_launch_rows(rng_gen *g, rngi::RowsLaunch &a, const rngi::LaunchShape &sh
   rngi::LaunchShape base = shape;
   if (!device_out) {
     base.bulk_auto = false;
-    base.bulk_forced = rngi::BulkChoice{};
+    base.bulk_forced = false;
   }
-  const rngi::LaunchShape sh = rngi::resolve_shape(base, a);
+  // Never under capture: the second state array would be allocated, and a
+  // replay would not find the arrays swapped.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool may_band = !a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n &&
+                        cudaStreamIsCapturing(g->compute, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  const rngi::LaunchShape sh = rngi::resolve_shape(base, a, may_band);
   bool swap = false;
-  if (!a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n) {
+  if (may_band) {
     const uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
     if (br) {
-      int rc = setup_bands(g, a, br, true, &swap, err);
+      int rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
       if (rc) return rc;
     }
   }
@@ -779,6 +802,7 @@ void rng_destroy(rng_gen *g) {
   cudaFree(g->d_state);
   cudaFree(g->d_state2);
   cudaFree(g->d_jump);
+  cudaFree(g->d_jump_small);
   for (int b = 0; b < 2; ++b) {
     cudaFree(g->d_buf[b]);
     if (g->produced[b]) cudaEventDestroy(g->produced[b]);
@@ -992,7 +1016,9 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   rngi::SlicedPlan plan;
   if (!g->opts.values_per_thread && a.out_mode == 0) {
     plan = rngi::choose_sliced(g->n, iterations, g->device, !capturing);
-    if (plan.quantum_rows && !band_memory(g, !a.from_hash))
+    if (plan.quantum_rows &&
+        band_memory(g, static_cast<uint32_t>((iterations + plan.quantum_rows - 1) / plan.quantum_rows), !a.from_hash) !=
+            cudaSuccess)
       plan = rngi::choose_sliced(g->n, iterations, g->device, false);
   }
   if (plan.blocks) {
@@ -1012,7 +1038,7 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
     uint64_t br = rngi::choose_band_rows(g->n, iterations, sh, g->device, true, a.out_mode);
     if (!br && !capturing) {
       br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
-      if (br && !band_memory(g, !a.from_hash)) br = 0;
+      if (br && band_memory(g, static_cast<uint32_t>((iterations + br - 1) / br), !a.from_hash) != cudaSuccess) br = 0;
     }
     if (br) {
       rc = setup_bands(g, a, br, !a.from_hash, &swap, err);

@@ -28,10 +28,14 @@ const void *rows_kernel_fn(uint32_t vpt, int width, int policy, uint32_t block, 
 // 4, 6 or 8 values per thread, 256-thread blocks.
 const void *rows_staged_kernel_fn(uint32_t vpt, bool banded, uint32_t out);
 // Row kernel whose rows are written by TMA bulk copies from `nb` shared
-// buffers (2 or 4 values per thread with 8 buffers, 8 with 4 or 8, 16 with
+// buffers (4 values per thread with 8 buffers, 8 with 12, 16 with 6, 24 with
 // 4; 256-thread blocks), and its dynamic shared memory in bytes.
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out);
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb);
+// Banded row kernel of few streams (at most 256 * vpt; vpt 1, 2, 4, 8 or 16):
+// several rows per bulk copy.
+const void *rows_multi_kernel_fn(uint32_t vpt, uint32_t out);
+size_t rows_multi_smem_bytes();
 const void *checksum_kernel_fn(uint32_t vpt, bool banded = false, uint32_t out = 0);
 // Bit-sliced generate-and-checksum kernel (output mode 0; checksum_sliced.cu):
 // blocks of kSlicedBlock threads, tiles of kSlicedTile streams.
@@ -76,13 +80,19 @@ struct RowsLaunch {
   const uint64_t *jump; // bands: nibble tables of M^(band * band_rows), band = 0, 1, ... (kJumpTableWords each)
   uint64_t *state_out;  // where final states go (== state unless banded)
   uint32_t out_mode;    // value emitted per state: 0 the state, 1 xorshift64* (selects the kernel)
+  uint32_t tile_w;      // streams per tile of the bulk-copy row kernel
+  uint32_t pace;        // bulk-copy kernels: 2^-20 ns per byte between a block's copies, or 0
 };
 
-// Values per thread and row buffers of the bulk-copy row kernel (nb == 0:
-// not used).
-struct BulkChoice {
-  uint32_t vpt = 0;
-  uint32_t nb = 0;
+// One launch on the bulk-copy kernels (nb == 0: not used).
+struct BulkPlan {
+  uint32_t vpt = 0;        // values per thread
+  uint32_t nb = 0;         // row buffers
+  uint32_t tile_w = 0;     // streams per tile (at most 256 * vpt)
+  bool multi = false;      // rows_multi_kernel: the whole row in one tile
+  uint64_t band_rows = 0;  // rows per band, or 0: not banded
+  uint32_t blocks = 0;     // persistent blocks, or 0: one per unit
+  uint32_t pace = 0;       // RowsLaunch::pace
 };
 
 struct LaunchShape {
@@ -91,10 +101,11 @@ struct LaunchShape {
   uint32_t grid;
   uint32_t width;         // widest store in values (1, 2, 4) the shape may use
   bool staged = false;    // rows off the 128-byte lines: the staged row kernel
-  bool bulk_auto = false;  // resolve_shape may pick the bulk-copy kernel for each launch
-  BulkChoice bulk_forced;  // store_policy 2: this bulk-copy shape for every device row
-  uint32_t sms = 0;        // SMs of the device the shape is for
-  uint32_t bulk_nb = 0;    // set by resolve_shape: this launch runs the bulk kernel (vpt values per thread)
+  bool direct = false;    // register stores also for rows off the lines
+  bool bulk_auto = false;   // resolve_shape may pick a bulk-copy kernel for each launch
+  bool bulk_forced = false; // store_policy 2: bulk copies for every device row, vpt values per thread
+  uint32_t sms = 0;         // SMs of the device the shape is for
+  BulkPlan bulk;            // set by resolve_shape: what this launch runs
 };
 
 // What one row-kernel launch ran (rng_launch_info without struct_size).
@@ -116,7 +127,8 @@ LaunchShape rows_shape(uint64_t streams, uint32_t vpt, uint32_t block, int devic
 // The shape one launch with output a.out runs: the bulk-copy kernel when
 // the shape names one for the alignment of a.out's rows (device outputs
 // only: the caller passes no host destination here), else `sh` as chosen.
-LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a);
+// may_band: whether this launch's rows may be split into bands.
+LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a, bool may_band);
 // store_policy: 0 default, 1 streaming (.cs), 2 bulk copies.  Register
 // stores are the widest of sh.width and what the output's alignment allows.
 // `sh` must come from resolve_shape.  info (optional) receives what ran.

@@ -205,6 +205,38 @@ __device__ __forceinline__ void bulk_wait_read() {
 // Waits until all of this thread's groups are complete (their writes done).
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+// Issue times of a block's bulk copies.  One SM can write 32 bytes a clock
+// (62 GB/s), so from about 130 of the 152 SMs on they offer more than HBM
+// takes (7.6-7.8 TB/s), and past that point it takes less: 6.3-6.7 TB/s,
+// whatever the pieces' size, order or number in flight.  Each block
+// therefore holds its copies to its share of a rate just under the ceiling,
+// by the global timer (32 ns steps, independent of the SM clock): 16 KiB per
+// SM every 316-324 ns wrote 7.65-7.79 TB/s in a copy-only kernel (memset
+// 7.58), 310 ns 7.1-7.3, unpaced 6.66.
+struct Pacer {
+  uint64_t t0 = 0;   // when the schedule began (ns)
+  uint64_t due = 0;  // since then (2^-20 ns)
+  // The time, to be read before the block's barrier so that its latency is
+  // not in the way of the copy.
+  static __device__ __forceinline__ uint64_t now() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+  }
+  // Waits for the turn of copies of `bytes`, `t` being a reading of now();
+  // rate: 2^-20 ns per byte, 0 = no schedule.  A block that is late by more
+  // than a microsecond (a new tile's states were loaded) goes on from there
+  // instead of catching up in a burst.
+  __device__ __forceinline__ void wait(uint64_t t, uint32_t bytes, uint32_t rate) {
+    if (!rate) return;
+    if (!t0) t0 = t;
+    const uint64_t turn = t0 + (due >> 20);
+    for (int polls = 0; polls < 4096 && t < turn; ++polls) t = now();
+    if (t > turn + 1024) t0 += t - turn - 1024;
+    due += static_cast<uint64_t>(bytes) * rate;
+  }
+};
+
 // Shared words of the bulk row kernel: NB row buffers of one tile plus two
 // words (a row whose segment starts on an odd word is staged one word
 // further on, so that its 16-byte-aligned body is 16-byte aligned in shared
@@ -219,16 +251,17 @@ __host__ __device__ constexpr int bulk_words() {
 // rows this block has staged, up to NB; both continue across the block's
 // tiles), one barrier per row, then one thread
 // issues a bulk copy of the row segment's 16-byte-aligned body and plain
-// 8-byte stores of an odd head or tail.  The SMs' store path then carries
-// only shared-memory writes.  A buffer is refilled only after the copy that
-// read it NB rows earlier has finished reading.  Values past `span` are
-// staged but not copied.  ring != 0: rows wrap around a ring of `ring` rows.
-// Every thread of the block must call it; the issuing thread must wait for
-// its groups (bulk_wait_all) before the block exits.
+// 8-byte stores of an odd head or tail, at the time the pacer gives.  The
+// SMs' store path then carries only shared-memory writes.  A buffer is
+// refilled only after the copy that read it NB rows earlier has finished
+// reading.  Values past `span` are staged but not copied.  ring != 0: rows
+// wrap around a ring of `ring` rows.  Every thread of the block must call
+// it; the issuing thread must wait for its groups (bulk_wait_all) before the
+// block exits.
 template <int VPT, int NB, int OUT = 0>
 __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *row, uint64_t pitch, uint64_t rows,
                                                uint64_t span, uint64_t ring, uint64_t *buf, uint32_t &kb,
-                                               uint32_t &warm) {
+                                               uint32_t &warm, Pacer &pacer, uint32_t pace) {
   static_assert(NB >= 2, "NB: at least 2");
   constexpr int kTile = kBlock * VPT;
   constexpr int kBuf = kTile + 2;
@@ -243,13 +276,18 @@ __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *ro
 #pragma unroll
     for (int v = 0; v < VPT; ++v) st[v] = prng::xorshift_update(st[v]);
     fence_proxy_async_smem();
-    // After this barrier the block fills the next buffer, last read by the
-    // copy issued NB - 1 rows before this one: at most NB - 2 later copies
-    // may still be reading.
-    if (threadIdx.x == 0 && warm + 1 >= NB) bulk_wait_read<NB - 2>();
+    uint64_t t = 0;
+    if (threadIdx.x == 0) {
+      if (pace) t = Pacer::now();
+      // After this barrier the block fills the next buffer, last read by the
+      // copy issued NB - 1 rows before this one: at most NB - 2 later copies
+      // may still be reading.
+      if (warm + 1 >= NB) bulk_wait_read<NB - 2>();
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
       const int body = (n - p) & ~1;
+      pacer.wait(t, 8u * static_cast<uint32_t>(n), pace);
       if (p) store_one<kPolicyStreaming>(row, b[1]);
       if ((n - p) & 1) store_one<kPolicyStreaming>(row + n - 1, b[p + n - 1]);
       if (body > 0) bulk_store(row + p, b + 2 * p, 8u * static_cast<uint32_t>(body));
@@ -369,34 +407,110 @@ __global__ void __launch_bounds__(kBlock) rows_staged_kernel(const RowsLaunch a)
 }
 
 // Row kernel whose rows are written by TMA bulk copies from shared memory
-// (emit_rows_bulk): the same work units as rows_staged_kernel, any row
-// alignment, and rings when unbanded.  The dynamic shared memory holds the
-// NB row buffers (bulk_words<VPT, NB>() words).
+// (emit_rows_bulk): work units as in rows_staged_kernel but for the tile's
+// width, any row alignment, and rings when unbanded.  A tile is a.tile_w <=
+// kBlock * VPT streams, chosen by the host so that the tiles come to whole
+// waves of the SMs (see bulk_plan); the threads' values past it are computed
+// and staged, not copied, which costs nothing here (the row loop waits for
+// HBM).  The dynamic shared memory holds the NB row buffers
+// (bulk_words<VPT, NB>() words).
 template <int VPT, int NB, bool BANDED, int OUT = 0>
 __global__ void __launch_bounds__(kBlock) rows_bulk_kernel(const RowsLaunch a) {
   extern __shared__ __align__(128) uint64_t bulk_buf[];
   const uint64_t span = a.s_end - a.s_begin;
-  constexpr uint64_t tile_vals = static_cast<uint64_t>(kBlock) * VPT;
-  const uint64_t n_tiles = (span + tile_vals - 1) / tile_vals;
+  const uint64_t n_tiles = (span + a.tile_w - 1) / a.tile_w;
   const uint64_t band_rows = BANDED ? a.band_rows : a.rows;
   const uint64_t n_bands = BANDED ? (a.rows + band_rows - 1) / band_rows : 1;
   uint32_t kb = 0, warm = 0;
+  Pacer pacer;
   for (uint64_t w = blockIdx.x; w < n_tiles * n_bands; w += gridDim.x) {
     const uint64_t tile = w % n_tiles;
     const uint64_t band = BANDED ? w / n_tiles : 0;
-    const uint64_t rel0 = tile * tile_vals;
+    const uint64_t rel0 = tile * a.tile_w;
+    const uint64_t end = span - rel0 < a.tile_w ? span : rel0 + a.tile_w;
     uint64_t st[VPT];
-    load_tile<VPT, 1>(st, a, rel0, span);
+    load_tile<VPT, 1>(st, a, rel0, end);
     if constexpr (BANDED) {
       __shared__ uint64_t jtab[16][16];
       if (band) jump_states<VPT>(st, a.jump, band, jtab);  // band is the same for the whole block
     }
     const uint64_t r0 = band * band_rows;
     const uint64_t rows = BANDED ? (a.rows - r0 < band_rows ? a.rows - r0 : band_rows) : a.rows;
-    emit_rows_bulk<VPT, NB, OUT>(st, a.out + r0 * a.pitch + rel0, a.pitch, rows, span - rel0,
-                                 BANDED ? 0 : a.ring_rows, bulk_buf, kb, warm);
+    emit_rows_bulk<VPT, NB, OUT>(st, a.out + r0 * a.pitch + rel0, a.pitch, rows, end - rel0,
+                                 BANDED ? 0 : a.ring_rows, bulk_buf, kb, warm, pacer, a.pace);
     if (a.write_state && band == n_bands - 1)
-      store_tile_state<VPT, 1>(st, BANDED ? a.state_out : a.state, a, rel0, span);
+      store_tile_state<VPT, 1>(st, BANDED ? a.state_out : a.state, a, rel0, end);
+  }
+  if (threadIdx.x == 0) bulk_wait_all();
+}
+
+// Few streams (at most kBlock * VPT, the whole row in every block) and many
+// rows, banded: R consecutive rows are one contiguous piece of the output
+// (pitch == streams), staged together and written by one bulk copy of up to
+// 32 KiB, where a row alone is too small a copy (4 KiB copies reached 4.2
+// TB/s).  NB pieces in turn, as in emit_rows_bulk.
+constexpr int kMultiBuffers = 6;
+
+template <int VPT, int R>
+__host__ __device__ constexpr int multi_words() {
+  return kMultiBuffers * (kBlock * VPT * R + 2);
+}
+
+template <int VPT, int R, int OUT = 0>
+__global__ void __launch_bounds__(kBlock) rows_multi_kernel(const RowsLaunch a) {
+  extern __shared__ __align__(128) uint64_t bulk_buf[];
+  __shared__ uint64_t jtab[16][16];
+  constexpr int kPiece = kBlock * VPT * R + 2;
+  const uint64_t span = a.s_end - a.s_begin;
+  const int n = static_cast<int>(span);
+  const uint64_t n_bands = (a.rows + a.band_rows - 1) / a.band_rows;
+  bool in[VPT];  // the thread's j-th value is a stream's
+#pragma unroll
+  for (int j = 0; j < VPT; ++j) in[j] = static_cast<int>(threadIdx.x) + kBlock * j < n;
+  uint32_t kb = 0, warm = 0;
+  Pacer pacer;
+  for (uint64_t band = blockIdx.x; band < n_bands; band += gridDim.x) {
+    uint64_t st[VPT];
+    load_tile<VPT, 1>(st, a, 0, span);
+    if (band) jump_states<VPT>(st, a.jump, band, jtab);
+    const uint64_t r0 = band * a.band_rows;
+    const uint64_t rows = a.rows - r0 < a.band_rows ? a.rows - r0 : a.band_rows;
+    uint64_t *row = a.out + r0 * span;
+    for (uint64_t r = 0; r < rows; r += R) {
+      const int m = rows - r < R ? static_cast<int>(rows - r) : R;
+      const int p = static_cast<int>((reinterpret_cast<uintptr_t>(row) >> 3) & 1);
+      uint64_t *b = bulk_buf + kb * kPiece;
+      uint64_t *d = b + p + threadIdx.x;
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (q < m) {
+#pragma unroll
+          for (int j = 0; j < VPT; ++j) {
+            if (in[j]) d[kBlock * j] = prng::emitted<OUT>(st[j]);
+            st[j] = prng::xorshift_update(st[j]);
+          }
+          d += n;
+        }
+      fence_proxy_async_smem();
+      uint64_t t = 0;
+      if (threadIdx.x == 0) {
+        if (a.pace) t = Pacer::now();
+        if (warm + 1 >= kMultiBuffers) bulk_wait_read<kMultiBuffers - 2>();
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        const int count = m * n, body = (count - p) & ~1;
+        pacer.wait(t, 8u * static_cast<uint32_t>(count), a.pace);
+        if (p) store_one<kPolicyStreaming>(row, b[1]);
+        if ((count - p) & 1) store_one<kPolicyStreaming>(row + count - 1, b[p + count - 1]);
+        if (body > 0) bulk_store(row + p, b + 2 * p, 8u * static_cast<uint32_t>(body));
+        bulk_commit();
+      }
+      kb = kb + 1 == kMultiBuffers ? 0 : kb + 1;
+      if (warm < kMultiBuffers) ++warm;
+      row += static_cast<uint64_t>(m) * n;
+    }
+    if (a.write_state && band == n_bands - 1) store_tile_state<VPT, 1>(st, a.state_out, a, 0, span);
   }
   if (threadIdx.x == 0) bulk_wait_all();
 }
@@ -679,7 +793,8 @@ __global__ void __launch_bounds__(kBlock) batch_work_kernel(const BatchWork *__r
 constexpr uint64_t kBulkUnitRows = 16;
 
 template <int VPT, int NB>
-__device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *buf, uint32_t &kb, uint32_t &warm) {
+__device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *buf, uint32_t &kb, uint32_t &warm,
+                                                  Pacer &pacer, uint32_t pace) {
   if (w.rows < kBulkUnitRows) {
     if (warm) {
       if (threadIdx.x == 0) bulk_wait_read<0>();
@@ -704,7 +819,7 @@ __device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *
   a.ring_rows = 0;
   uint64_t st[VPT];
   load_tile<VPT, 1>(st, a, 0, w.count);
-  emit_rows_bulk<VPT, NB>(st, w.out + w.s_begin, w.streams, w.rows, w.count, 0, buf, kb, warm);
+  emit_rows_bulk<VPT, NB>(st, w.out + w.s_begin, w.streams, w.rows, w.count, 0, buf, kb, warm, pacer, pace);
 }
 
 template <int VPT, int NB>
@@ -713,10 +828,11 @@ __global__ void __launch_bounds__(kBlock) batch_work_bulk_kernel(const BatchWork
   extern __shared__ __align__(128) uint64_t bulk_buf[];
   static_assert(bulk_words<VPT, NB>() >= staged_words<VPT>(), "short units stage in the bulk buffers");
   uint32_t kb = 0, warm = 0;
+  Pacer pacer;
   if (counter == nullptr) {
     if (blockIdx.x < n) {
       const BatchWork w = work[blockIdx.x];
-      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm);
+      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm, pacer, 0);
     }
   } else {
     __shared__ uint32_t s_unit;
@@ -727,7 +843,7 @@ __global__ void __launch_bounds__(kBlock) batch_work_bulk_kernel(const BatchWork
       __syncthreads();
       if (u >= n) break;
       const BatchWork w = work[u];
-      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm);
+      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm, pacer, 0);
     }
   }
   if (threadIdx.x == 0) bulk_wait_all();
@@ -902,8 +1018,21 @@ template <bool BANDED, int OUT>
 const void *select_rows_bulk_t(uint32_t vpt, uint32_t nb) {
   if (vpt == 4 && nb == 8) return reinterpret_cast<const void *>(&rows_bulk_kernel<4, 8, BANDED, OUT>);
   if (vpt == 8 && nb == 12) return reinterpret_cast<const void *>(&rows_bulk_kernel<8, 12, BANDED, OUT>);
-  if (vpt == 16 && nb == 4) return reinterpret_cast<const void *>(&rows_bulk_kernel<16, 4, BANDED, OUT>);
+  if (vpt == 16 && nb == 6) return reinterpret_cast<const void *>(&rows_bulk_kernel<16, 6, BANDED, OUT>);
+  if (vpt == 24 && nb == 4) return reinterpret_cast<const void *>(&rows_bulk_kernel<24, 4, BANDED, OUT>);
   return nullptr;
+}
+
+template <int OUT>
+const void *select_rows_multi_t(uint32_t vpt) {
+  switch (vpt) {
+    case 1: return reinterpret_cast<const void *>(&rows_multi_kernel<1, 16, OUT>);
+    case 2: return reinterpret_cast<const void *>(&rows_multi_kernel<2, 8, OUT>);
+    case 4: return reinterpret_cast<const void *>(&rows_multi_kernel<4, 4, OUT>);
+    case 8: return reinterpret_cast<const void *>(&rows_multi_kernel<8, 2, OUT>);
+    case 16: return reinterpret_cast<const void *>(&rows_multi_kernel<16, 1, OUT>);
+    default: return nullptr;
+  }
 }
 
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out) {
@@ -911,6 +1040,11 @@ const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t
   if (out != 0) return nullptr;
   return banded ? select_rows_bulk_t<true, 0>(vpt, nb) : select_rows_bulk_t<false, 0>(vpt, nb);
 }
+
+const void *rows_multi_kernel_fn(uint32_t vpt, uint32_t out) {
+  return out == 1 ? select_rows_multi_t<1>(vpt) : out == 0 ? select_rows_multi_t<0>(vpt) : nullptr;
+}
+size_t rows_multi_smem_bytes() { return multi_words<16, 1>() * sizeof(uint64_t); }
 
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb) {
   return size_t(nb) * (size_t(kBlock) * vpt + 2) * sizeof(uint64_t);

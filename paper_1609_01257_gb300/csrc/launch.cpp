@@ -79,46 +79,113 @@ uint32_t bulk_buffers(uint32_t vpt) {
   switch (vpt) {
     case 4: return 8;
     case 8: return 12;
-    case 16: return 4;
+    case 16: return 6;
+    case 24: return 4;
     default: return 0;
   }
 }
 
-// Bulk-copy row kernel (values per thread, row buffers) for one launch of
-// `rows` rows over `streams` streams when the caller leaves the shape to the
-// library, for rows on 128-byte lines (`lined`) and off them; nb == 0: keep
-// the register or staged kernel.  Measured on GB300 (GB/s; the register-
-// store or staged kernel in brackets):
-//  - on the lines, 1024 rows: 2^22 streams 7517 at (8, 12) [7470]; below
-//    3.5 M streams the register kernels stay ahead (2^20: 7211 [7247]; 2^16:
-//    6574 [6858]);
-//  - off the lines, 1024 rows, at (8, 12): 2^22 + 1 streams 7125 [6957], an
-//    output one word off a line 7147 [6893], 3,000,017 streams 6983 [6713],
-//    250,001 7078 [5629], 65,537 (banded) 6343 [4957]; at (16, 4): 1,000,003
-//    streams 6769 [6333] (6565 at (8, 12));
-//  - off the lines, 16-128 rows: 3,000,017 streams at (8, 12) 6215-7121
-//    [6002-7107]; 250,001 streams 2917-6296 [2595-6250]; 65,537 streams
-//    (33 tiles of 2048) at (4, 8) 877-2312 [585-1730]; 1,000,003 streams
-//    staged stays level or ahead below 128 rows (6248-6494 at 64-96 rows
-//    against 6155-6443); at 8 rows every form is within ~10 %.
-// Each copy has a fixed cost: 4 KiB copies (two values per thread) stayed
-// near 4.2 TB/s, so bulk tiles hold 8 KiB and more.  With one block per SM
-// (the buffers take most of its shared memory) each tile's start -- loading
-// its states -- is exposed, so lined launches of few rows keep the register
-// kernels: 2^22 streams x 128 rows 7221 [7209], 2^24 x 32 rows 6574 [6580],
-// 2^26 x 8 rows 4852 [5368], 2^28 x 2 rows 2233 [3503].
-BulkChoice bulk_default(uint64_t streams, uint64_t rows, bool lined, uint32_t sms) {
-  const uint64_t M = uint64_t(1) << 20;
-  if (lined) return streams >= 7 * M / 2 && rows >= 128 ? BulkChoice{8, 12} : BulkChoice{};
-  if (streams < 64 * 1024 || rows < 16) return BulkChoice{};
-  if (streams >= M / 2 && streams < 2 * M) return rows >= 128 ? BulkChoice{16, 4} : BulkChoice{};
-  if (streams < M / 2 && rows < 256) {
-    // Unbanded (banding starts at 256 rows): when tiles of 2048 streams
-    // would leave most SMs idle, tiles of 1024 give twice as many blocks.
-    const uint64_t tiles8 = (streams + uint64_t(kGenBlock) * 8 - 1) / (uint64_t(kGenBlock) * 8);
-    if (tiles8 * 2 < sms) return BulkChoice{4, 8};
+namespace {
+
+// Blocks that write at the same time hold their copies to this rate (bytes a
+// second, all together): see Pacer.  With 152 blocks and 2^22 streams x 256
+// rows 7.5, 7.6, 7.7 and 7.8e12 gave 7422, 7518, 7621 and 7711 GB/s; a
+// copy-only kernel held 7.88e12 and fell back at 8.0e12.
+constexpr double kWriteRate = 7.7e12;
+
+uint32_t pace_of(uint64_t blocks) {
+  return static_cast<uint32_t>(static_cast<double>(blocks) / kWriteRate * 1e9 * 1048576.0);
+}
+
+uint32_t ceil16(uint64_t v) { return static_cast<uint32_t>((v + 15) / 16 * 16); }
+
+}  // namespace
+
+// The bulk-copy kernels for one launch of `rows` rows over `streams` streams
+// when the caller leaves the shape to the library, for rows on 128-byte lines
+// (`lined`) and off them; nb == 0: keep the register or staged kernels.
+// may_band: the rows may be split into bands; out_bytes: the output's size
+// (the ring's, when rows wrap).  One block per SM, all with equal shares:
+// tiles and bands come to whole rounds of the SMs, because a paced block does
+// not use what another leaves (1000003 streams x 512 rows, 16 values per
+// thread: 304 tiles of 3296 in two rounds 7555 GB/s, 245 of 4096 6106).  A
+// block's step per row takes about 0.3 us with 8 values per thread and 0.44
+// with 16, so tiles are as wide as the threads' values allow.
+// Where the lines lie (GB300, us before / with this plan):
+//  - up to 4096 streams, the whole row in a block: 300 x 100 44 / 14, 1001 x
+//    4096 60 / 18, 4096 x 65536 333 / 294; rows on the lines keep register
+//    stores below 256 MB (4096 x 4096 32 / 33) and 16 rows per band;
+//  - 5500 x 1024 74 / 24, 20001 x 16384 549 / 359, 65537 x 255 58 / 35, 131073
+//    x 1024 188 / 154; below 128 rows register stores (direct_vpt) are faster;
+//  - 250001 x 255 81 / 82 (in bands 82), x 1024 293 / 281: from 1024 rows;
+//  - 400001 x 64 51 / 41, 1000003 x 128 167 / 150, 3000017 x 128 453 / 428, 2^22
+//    + 1 x 64 317 / 306; at 16 rows even or worse;
+//  - on the lines, 2^20 x 255 307 / 292, 2^22 x 128 602 / 584, 65536 x 4096 293 /
+//    294 (and 340 where 128 unpaced SMs are past the ceiling); 2^22 x 64 308 /
+//    324, 2^24 x 32 656 / 690 (each tile's loads are exposed).
+BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, uint64_t out_bytes, uint32_t sms) {
+  constexpr uint64_t M = uint64_t(1) << 20;
+  BulkPlan p;
+  const uint64_t bytes = 8 * streams * rows;
+  uint64_t units;
+  if (streams <= 4096) {
+    if (!may_band || rows < (lined ? 16 * uint64_t(sms) : 64)) return p;
+    if (lined && streams > 1024 && bytes < 256 * M) return p;
+    const uint64_t bands = std::min<uint64_t>(sms, rows / 16);
+    p.multi = true;
+    p.vpt = 1;
+    while (streams > uint64_t(kGenBlock) * p.vpt) p.vpt *= 2;
+    p.nb = 6;
+    p.tile_w = static_cast<uint32_t>(streams);
+    p.band_rows = (rows + bands - 1) / bands;
+    units = (rows + p.band_rows - 1) / p.band_rows;
+  } else {
+    const bool many = streams >= 7 * M / 2;
+    // One tile of 24 values per thread rather than two half empty ones of 16.
+    p.vpt = streams <= uint64_t(kGenBlock) * 24 ? 24 : 16;
+    p.nb = bulk_buffers(p.vpt);
+    const uint64_t most = uint64_t(kGenBlock) * p.vpt;
+    const uint64_t tiles = (streams + most - 1) / most;
+    if (lined) {
+      if (many ? rows < 128 : rows <= 128 || bytes < (tiles < sms ? 1024 : 256) * M) return BulkPlan{};
+    } else if (rows < (streams < uint64_t(sms) * 1024 ? 128 : many ? 16 : 32)) {
+      return BulkPlan{};
+    }
+    const bool narrow = tiles < sms && tiles > sms / 4 && rows < 1024 && streams <= uint64_t(sms) * 2048;
+    if (rows < 32 || narrow) {
+      // Few rows of many streams: one block per tile, so that a tile's last
+      // copies and the next one's start overlap (2^22 + 1 x 16 103, register
+      // stores 123).  Fewer tiles than SMs, too many for bands that are worth
+      // their jumps: the narrowest tiles whose copies are not too small.
+      p.vpt = 8;
+      p.nb = bulk_buffers(p.vpt);
+      p.tile_w = kGenBlock * 8;
+      return p;
+    }
+    uint64_t bands = 1;
+    if (tiles >= sms) {
+      const uint64_t rounds = (tiles + sms - 1) / sms;
+      p.tile_w = ceil16((streams + rounds * sms - 1) / (rounds * sms));
+    } else {
+      if (may_band) bands = std::max<uint64_t>(1, std::min<uint64_t>(sms / tiles, rows / 16));
+      p.tile_w = ceil16((streams + sms / bands - 1) / (sms / bands));
+      if (bands > 1) p.band_rows = (rows + bands - 1) / bands;
+    }
+    units = (streams + p.tile_w - 1) / p.tile_w * (bands > 1 ? (rows + p.band_rows - 1) / p.band_rows : 1);
   }
-  return BulkChoice{8, 12};
+  p.blocks = static_cast<uint32_t>(std::min<uint64_t>(units, sms));
+  // Outputs that the 129 MB L2 can take are written as fast as it takes them.
+  if (out_bytes >= 128 * M) p.pace = pace_of(p.blocks);
+  return p;
+}
+
+// Rows off the lines without a bulk plan (small launches): register stores
+// all the same when the staged kernel would have few blocks, each with a
+// barrier per row.  GB300, staged / direct us: 65537 x 16 14.3 / 6.5, x 64
+// 39 / 12; 20001 x 100 59 / 12; 131073 x 64 39 / 16; 250001 x 16 11.9 / 9.8.
+uint32_t direct_vpt(uint64_t streams) {
+  if (streams >= 384 * 1024) return 0;
+  return streams >= 100 * 1024 ? 4 : streams >= 64 * 1024 ? 2 : 1;
 }
 
 LaunchShape rows_shape(uint64_t streams, uint32_t vpt, uint32_t block, int device, uint32_t max_grid,
@@ -129,12 +196,12 @@ LaunchShape rows_shape(uint64_t streams, uint32_t vpt, uint32_t block, int devic
   if (policy == kStoreBulk) {
     // Every row written by bulk copies, whatever its alignment.
     sh.vpt = vpt ? vpt : 8;
-    sh.bulk_forced = BulkChoice{sh.vpt, bulk_buffers(sh.vpt)};
+    sh.bulk_forced = bulk_buffers(sh.vpt) != 0;
     sh.width = 1;
     const uint64_t tiles = (streams + uint64_t(kGenBlock) * sh.vpt - 1) / (uint64_t(kGenBlock) * sh.vpt);
     uint64_t grid = max_grid && max_grid < tiles ? max_grid : tiles;
     if (grid > 0x7fffffffull) grid = 0x7fffffffull;
-    sh.grid = sh.bulk_forced.nb && sh.block == kGenBlock ? static_cast<uint32_t>(grid ? grid : 1) : 0;
+    sh.grid = sh.bulk_forced && sh.block == kGenBlock ? static_cast<uint32_t>(grid ? grid : 1) : 0;
     return sh;
   }
   sh.bulk_auto = policy == kStoreStreaming && vpt == 0 && sh.block == kGenBlock && max_grid == 0 && width == 0;
@@ -178,23 +245,37 @@ LaunchShape rows_shape(uint64_t streams, uint32_t vpt, uint32_t block, int devic
   return sh;
 }
 
-LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a) {
+LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a, bool may_band) {
   LaunchShape r = sh;
-  r.bulk_nb = 0;
+  r.bulk = BulkPlan{};
   if (!a.out) return r;
+  const uint64_t span = a.s_end - a.s_begin;
   const bool lined = a.pitch % 16 == 0 && reinterpret_cast<uintptr_t>(a.out) % 128 == 0;
-  const BulkChoice c = sh.bulk_forced.nb ? sh.bulk_forced
-                       : sh.bulk_auto    ? bulk_default(a.s_end - a.s_begin, a.rows, lined, sh.sms)
-                                         : BulkChoice{};
-  if (!c.nb) return r;
-  r.vpt = c.vpt;
-  r.bulk_nb = c.nb;
+  if (sh.bulk_forced) {
+    r.bulk.vpt = sh.vpt;
+    r.bulk.nb = bulk_buffers(sh.vpt);
+    r.bulk.tile_w = kGenBlock * sh.vpt;
+  } else if (sh.bulk_auto) {
+    r.bulk = bulk_plan(span, a.rows, lined, may_band,
+                       8 * span * (a.ring_rows && a.ring_rows < a.rows ? a.ring_rows : a.rows), sh.sms);
+  }
+  if (!r.bulk.nb) {
+    const uint32_t v = sh.bulk_auto && !lined ? direct_vpt(span) : 0;
+    if (v) {
+      r.direct = true;
+      r.staged = false;
+      r.vpt = v;
+      r.width = 2;
+      r.grid = static_cast<uint32_t>((span + uint64_t(kGenBlock) * v - 1) / (uint64_t(kGenBlock) * v));
+    }
+    return r;
+  }
+  r.vpt = r.bulk.vpt;
   r.staged = false;
   r.width = 1;
-  const uint64_t span = a.s_end - a.s_begin;
-  const uint64_t tiles = (span + uint64_t(kGenBlock) * c.vpt - 1) / (uint64_t(kGenBlock) * c.vpt);
+  const uint64_t tiles = (span + r.bulk.tile_w - 1) / r.bulk.tile_w;
   uint64_t grid = tiles;
-  if (sh.vpt == c.vpt && sh.grid && sh.grid < tiles) grid = sh.grid;  // a grid the caller asked for
+  if (sh.bulk_forced && sh.grid && sh.grid < tiles) grid = sh.grid;  // a grid the caller asked for
   if (grid > 0x7fffffffull) grid = 0x7fffffffull;
   r.grid = static_cast<uint32_t>(grid ? grid : 1);
   return r;
@@ -202,7 +283,7 @@ LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a) {
 
 cudaError_t launch_rows(const RowsLaunch &a, const LaunchShape &sh, int store_policy, cudaStream_t st,
                         LaunchInfo *info) {
-  if (a.band_rows && (a.ring_rows || !a.jump || (a.write_state && a.state_out == a.state)))
+  if (a.band_rows && (a.ring_rows || !a.jump || (a.write_state && !a.from_hash && a.state_out == a.state)))
     return cudaErrorInvalidValue;
   // Widest store the output's alignment allows: every row must start on an
   // 8*W-byte boundary (pitch a multiple of W, base aligned to 8*W bytes).
@@ -222,11 +303,13 @@ cudaError_t launch_rows(const RowsLaunch &a, const LaunchShape &sh, int store_po
   // pieces; the tiles are the same.
   const uint32_t vpt = sh.vpt;
   const bool small_vpt = vpt == 1 || vpt == 2 || vpt == 4 || vpt == 6 || vpt == 8;
-  const bool bulk = a.out && sh.bulk_nb;
-  const bool staged = !bulk && a.out && !a.ring_rows && sh.block == kGenBlock && small_vpt &&
+  const bool bulk = a.out && sh.bulk.nb;
+  const bool staged = !bulk && !sh.direct && a.out && !a.ring_rows && sh.block == kGenBlock && small_vpt &&
                       (sh.staged || a.pitch % 16 != 0 || base % 128 != 0);
   const int policy = store_policy == kStoreBulk ? kStoreStreaming : store_policy;
-  const void *fn = bulk     ? rows_bulk_kernel_fn(vpt, sh.bulk_nb, a.band_rows != 0, a.out_mode)
+  const void *fn = bulk && sh.bulk.multi
+                       ? (a.band_rows && a.pitch == a.s_end - a.s_begin ? rows_multi_kernel_fn(vpt, a.out_mode) : nullptr)
+                   : bulk   ? rows_bulk_kernel_fn(vpt, sh.bulk.nb, a.band_rows != 0, a.out_mode)
                    : staged ? rows_staged_kernel_fn(vpt, a.band_rows != 0, a.out_mode)
                             : rows_kernel_fn(vpt, width, policy, sh.block, a.band_rows != 0, a.out_mode);
   uint64_t grid = sh.grid;
@@ -234,18 +317,22 @@ cudaError_t launch_rows(const RowsLaunch &a, const LaunchShape &sh, int store_po
   if (!fn) return cudaErrorInvalidValue;
   size_t smem = 0;
   if (bulk) {
-    smem = rows_bulk_smem_bytes(vpt, sh.bulk_nb);
+    smem = sh.bulk.multi ? rows_multi_smem_bytes() : rows_bulk_smem_bytes(vpt, sh.bulk.nb);
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
   RowsLaunch args = a;
+  const uint64_t tile_w = bulk ? sh.bulk.tile_w : uint64_t(sh.block) * vpt;
+  args.tile_w = static_cast<uint32_t>(tile_w);
+  args.pace = bulk ? sh.bulk.pace : 0;
   void *params[] = {&args};
   if (a.band_rows) {
     // One block per (tile, band) unit, unless the shape asked for fewer.
-    const uint64_t tiles = (span + uint64_t(sh.block) * vpt - 1) / (uint64_t(sh.block) * vpt);
+    const uint64_t tiles = (span + tile_w - 1) / tile_w;
     const uint64_t units = tiles * ((a.rows + a.band_rows - 1) / a.band_rows);
     if (grid >= tiles) grid = units < 0x7fffffffull ? units : 0x7fffffffull;
   }
+  if (bulk && sh.bulk.blocks && sh.bulk.blocks < grid) grid = sh.bulk.blocks;
   if (grid > 0x7fffffffull) grid = 0x7fffffffull;
   cudaError_t e = cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(sh.block), params, smem, st);
   if (e == cudaSuccess) {
@@ -255,7 +342,7 @@ cudaError_t launch_rows(const RowsLaunch &a, const LaunchShape &sh, int store_po
       info->vpt = vpt;
       info->block = sh.block;
       info->grid = static_cast<uint32_t>(grid);
-      info->row_buffers = bulk ? sh.bulk_nb : 0;
+      info->row_buffers = bulk ? sh.bulk.nb : 0;
       info->band_rows = a.band_rows;
     }
   }
@@ -303,8 +390,9 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
   const uint64_t sms = static_cast<uint64_t>(device_sm_count(device));
   const uint64_t tiles = (streams + uint64_t(sh.block) * sh.vpt - 1) / (uint64_t(sh.block) * sh.vpt);
   const uint64_t min_band = checksum ? 64 : 128;
+  if (!checksum && sh.bulk.nb && !sh.bulk_forced) return sh.bulk.band_rows;  // part of the plan
   const void *fn = checksum     ? checksum_kernel_fn(sh.vpt, true, out)
-                   : sh.bulk_nb ? rows_bulk_kernel_fn(sh.vpt, sh.bulk_nb, true, out)
+                   : sh.bulk.nb ? rows_bulk_kernel_fn(sh.vpt, sh.bulk.nb, true, out)
                    : sh.staged  ? rows_staged_kernel_fn(sh.vpt, true, out)
                                 : rows_kernel_fn(sh.vpt, 1, kStoreStreaming, sh.block, true, out);
   if (!fn || rows < 2 * min_band) return 0;  // no banded variant of this shape, or too few rows
@@ -351,10 +439,12 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
   // bound by one block's rows, one after another, so they take fewer values
   // per thread and more blocks (us on GB300 at 4 / 8 / 16: 8192 x 1024 25 / 30
   // / 40; 65536 x 256 32 / 31 / 40; 1000003 x 16 37 / 27 / 29; 262144 x 256
-  // 62 / 62 / 60; 65536 x 4096 176 / 167 / 173).  A tile that would be mostly
-  // past the end of the streams is halved.
+  // 62 / 62 / 60; 65536 x 4096 176 / 167 / 173) unless there are many tiles
+  // anyway.  A tile that would be mostly past the end of the streams is halved.
   const uint64_t values = span * rows;
-  uint32_t v = values >= (uint64_t(1) << 26) ? 16 : values >= (uint64_t(1) << 24) ? 8 : 4;
+  uint32_t v = values >= (uint64_t(1) << 26)                              ? 16
+               : values >= (uint64_t(1) << 24) || span >= 256 * 8 * 152 ? 8
+                                                                          : 4;
   while (v > 1) {
     const uint64_t tile = uint64_t(kGenBlock) * v, tiles = (span + tile - 1) / tile;
     if (span * 5 >= tiles * tile * 4) break;
