@@ -490,12 +490,11 @@ void rng_batch_destroy(rng_batch *b);
  *
  * It produces exactly what rng_batch_create + rng_batch_run produce for the
  * same instances (iterations 0 .. iterations[k]-1 of instance k into outs[k],
- * iteration-major), with one launch of the served form's work-list kernel
- * (an instance table, a unit table and a work counter), but it allocates
- * nothing: no cudaMalloc, cudaFree, pinned or host heap memory and no CUDA
- * graph.  Its scratch -- the counter and the two tables -- is one fixed array
- * of RNG_NOALLOC_SCRATCH_BYTES in device global memory that every GPU loading
- * this library holds until the process exits.
+ * iteration-major) with one launch, but it allocates nothing: no cudaMalloc,
+ * cudaFree, pinned or host heap memory and no CUDA graph.  Up to 64 instances
+ * are passed to the kernel as its parameters; the table of more is uploaded
+ * to one fixed array of RNG_NOALLOC_SCRATCH_BYTES in device global memory that
+ * every GPU loading this library holds until the process exits.
  *
  * Limits: at most RNG_NOALLOC_MAX_INSTANCES instances and
  * RNG_NOALLOC_MAX_UNITS work units, one unit per started group of 2048
@@ -506,25 +505,24 @@ void rng_batch_destroy(rng_batch *b);
  * Arguments are those of rng_batch_create (host arrays of `count` entries;
  * outs[k] caller-owned device memory of 8*streams[k]*iterations[k] bytes,
  * 8-byte aligned); `stream` is the cudaStream_t to launch on (NULL = the
- * legacy default stream).  The call queues a table upload, a reset of the
- * counter and the kernel on `stream` and returns without waiting for the
- * kernel.  The tables are uploaded from pageable host memory, so the call
- * may wait for work already queued on `stream` before it returns.
+ * legacy default stream).  The call queues the kernel (above 64 instances,
+ * after a table upload) on `stream` and returns without waiting for it.  The
+ * table is uploaded from pageable host memory, so a call with more than 64
+ * instances may wait for work already queued on `stream` before it returns.
  *
  * The first call on a device, with that device current, looks up the
  * scratch array's device address (cudaGetSymbolAddress) and caches it; this
  * may make the driver load the library's device code.  Make that first call
  * before any stream capture begins.  A cudaDeviceReset destroys the array with
  * the context, so do not call this entry point again on a device after
- * resetting it in the same process.  All calls share the one array and each
- * call overwrites it, so calls whose work overlaps on the GPU (launched on
+ * resetting it in the same process.  Calls with more than 64 instances share
+ * the one array and each overwrites it, so such calls whose work overlaps on the GPU (launched on
  * different streams without ordering between them) race and produce wrong
  * output; calls on one stream are ordered and safe.  The host side of
  * concurrent calls is serialised by a lock. */
 #define RNG_NOALLOC_MAX_INSTANCES 4096u
 #define RNG_NOALLOC_MAX_UNITS 262144u
-#define RNG_NOALLOC_SCRATCH_BYTES \
-    (256u + RNG_NOALLOC_MAX_INSTANCES * 48u + RNG_NOALLOC_MAX_UNITS * 16u)
+#define RNG_NOALLOC_SCRATCH_BYTES (RNG_NOALLOC_MAX_INSTANCES * 52u)
 int rng_batch_generate_noalloc(uint32_t count, const uint64_t *streams,
                                const uint64_t *iterations, const uint64_t *seeds,
                                uint64_t *const *outs, void *stream, rng_err **err);

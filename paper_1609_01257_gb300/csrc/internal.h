@@ -48,6 +48,7 @@ const void *batch_work_kernel_fn(uint32_t vpt);
 // (8, 6) or (8, 12) values per thread and row buffers; dynamic shared memory
 // rows_bulk_smem_bytes(vpt, nb).
 const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb);
+const void *noalloc_kernel_fn();
 const void *init_kernel_fn();
 const void *copy_kernel_fn();
 const void *zero_pair_kernel_fn();
@@ -193,6 +194,21 @@ struct BatchInstance {
   uint32_t from_hash;
   uint32_t write_state;
 };
+// Allocation-free form: `count` instances, first[k] the number of tiles of
+// 256 * kNoallocVpt streams before instance k's.  Up to kNoallocFew instances
+// travel with the launch (inst == nullptr: few, few_first), more in device
+// memory.
+constexpr uint32_t kNoallocVpt = 4;
+constexpr uint32_t kNoallocFew = 64;
+struct NoallocArgs {
+  const BatchInstance *inst;
+  const uint32_t *first;
+  uint32_t count;
+  uint32_t few_first[kNoallocFew];
+  BatchInstance few[kNoallocFew];
+};
+static_assert(sizeof(NoallocArgs) <= 4096, "kernel parameters");
+cudaError_t launch_noalloc(const NoallocArgs &args, uint32_t tiles, cudaStream_t st);
 struct BatchUnit {
   uint32_t inst;
   uint32_t count;   // streams in this unit (<= tile)

@@ -576,6 +576,13 @@ cudaError_t launch_batch_work(const BatchWork *work, uint32_t n, uint32_t *count
   return e;
 }
 
+cudaError_t launch_noalloc(const NoallocArgs &args, uint32_t tiles, cudaStream_t st) {
+  void *params[] = {const_cast<NoallocArgs *>(&args)};
+  const cudaError_t e = cudaLaunchKernel(noalloc_kernel_fn(), dim3(tiles), dim3(kGenBlock), params, 0, st);
+  if (e == cudaSuccess) count_launch();
+  return e;
+}
+
 cudaError_t launch_batch(const BatchInstance *inst, const BatchUnit *units, uint32_t n_units,
                          uint32_t *counter, uint32_t vpt, uint32_t block, uint32_t grid,
                          cudaStream_t st) {

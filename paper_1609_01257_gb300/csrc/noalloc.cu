@@ -5,12 +5,12 @@
 // framework whose memory pool owns the whole device and forbids allocations
 // beside it, or latency-bound callers that must not pay for an allocation
 // (and the device-wide synchronisation a cudaFree implies) on every call.
-// This entry point produces the batched form's output with the served form's
-// work-list kernel (worklist_kernel: an instance table, a unit table and a
-// work counter), whose scratch -- the counter and the two tables, 48 bytes
-// per instance and 16 per unit -- lives in one fixed-size array in device
-// global memory declared at file scope below.  Every GPU that loads the
-// library holds this array until the process exits.
+// This entry point produces the batched form's output with one launch of
+// noalloc_kernel, whose blocks find their tile from the instance table alone.
+// Up to 64 instances are kernel parameters; more are uploaded to one
+// fixed-size array in device global memory declared at file scope below (52
+// bytes per instance).  Every GPU that loads the library holds this array
+// until the process exits.
 //
 // Host code cannot use the array's name as a device address (it names a
 // host-side stand-in), so the address is looked up with
@@ -27,25 +27,26 @@
 
 namespace {
 
-constexpr uint32_t kVpt = 8;
-constexpr uint32_t kBlock = 256;
-constexpr uint64_t kTile = uint64_t(kBlock) * kVpt;
-constexpr size_t kCounterBytes = 256;
+constexpr uint64_t kUnit = 2048;  // streams of one work unit, in which the limit is counted
+constexpr uint64_t kTile = uint64_t(rngi::kGenBlock) * rngi::kNoallocVpt;
 constexpr size_t kInstBytes = size_t(RNG_NOALLOC_MAX_INSTANCES) * sizeof(rngi::BatchInstance);
-constexpr size_t kUnitBytes = size_t(RNG_NOALLOC_MAX_UNITS) * sizeof(rngi::BatchUnit);
-constexpr size_t kScratchBytes = kCounterBytes + kInstBytes + kUnitBytes;
+constexpr size_t kScratchBytes = kInstBytes + size_t(RNG_NOALLOC_MAX_INSTANCES) * sizeof(uint32_t);
 constexpr int kMaxDevices = 64;
 
-static_assert(sizeof(rngi::BatchInstance) == 48 && sizeof(rngi::BatchUnit) == 16, "table entry sizes");
-static_assert(kInstBytes % 256 == 0, "unit table must stay 256-byte aligned");
+static_assert(sizeof(rngi::BatchInstance) == 48, "table entry size");
 static_assert(RNG_NOALLOC_SCRATCH_BYTES == kScratchBytes, "header and scratch size disagree");
 
-// Scratch: [work counter | instance table | unit table].
+// Scratch: [instance table | first tile of each instance].
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-// Host staging for the tables (no host allocation per call either).
-rngi::BatchInstance g_host_inst[RNG_NOALLOC_MAX_INSTANCES];
-rngi::BatchUnit g_host_units[RNG_NOALLOC_MAX_UNITS];
+// Host staging (no host allocation per call either): the instances' order and
+// the tables of a call with many.
+uint32_t g_order[RNG_NOALLOC_MAX_INSTANCES];
+struct HostTable {
+  rngi::BatchInstance inst[RNG_NOALLOC_MAX_INSTANCES];
+  uint32_t first[RNG_NOALLOC_MAX_INSTANCES];
+} g_host;
+static_assert(sizeof(HostTable) == kScratchBytes, "one upload");
 
 std::mutex g_mu;  // serialises the host side of calls (staging arrays, address cache)
 unsigned char *g_scratch_addr[kMaxDevices];
@@ -68,12 +69,12 @@ extern "C" int rng_batch_generate_noalloc(uint32_t count, const uint64_t *stream
       return rngi::fail(err, RNG_EINVAL, "rng_batch_generate_noalloc: instance %u output size overflows", k);
     if (reinterpret_cast<uintptr_t>(outs[k]) % 8)
       return rngi::fail(err, RNG_EINVAL, "rng_batch_generate_noalloc: instance %u output not 8-byte aligned", k);
-    n_units += (streams[k] + kTile - 1) / kTile;
+    n_units += (streams[k] + kUnit - 1) / kUnit;
   }
   if (n_units > RNG_NOALLOC_MAX_UNITS)
     return rngi::fail(err, RNG_EINVAL,
                       "rng_batch_generate_noalloc: %llu work units (tiles of %llu streams), at most %u",
-                      (unsigned long long)n_units, (unsigned long long)kTile, RNG_NOALLOC_MAX_UNITS);
+                      (unsigned long long)n_units, (unsigned long long)kUnit, RNG_NOALLOC_MAX_UNITS);
 
   std::lock_guard<std::mutex> lk(g_mu);
   int dev = 0;
@@ -88,14 +89,21 @@ extern "C" int rng_batch_generate_noalloc(uint32_t count, const uint64_t *stream
     if (st != cudaSuccess) return rngi::cuda_fail(err, st, "rng_batch_generate_noalloc: cudaGetSymbolAddress");
     g_scratch_addr[dev] = static_cast<unsigned char *>(p);
   }
-  unsigned char *base = g_scratch_addr[dev];
-  uint32_t *d_counter = reinterpret_cast<uint32_t *>(base);
-  rngi::BatchInstance *d_inst = reinterpret_cast<rngi::BatchInstance *>(base + kCounterBytes);
-  rngi::BatchUnit *d_units = reinterpret_cast<rngi::BatchUnit *>(base + kCounterBytes + kInstBytes);
 
-  uint32_t u = 0;
-  for (uint32_t k = 0; k < count; ++k) {
-    rngi::BatchInstance &in = g_host_inst[k];
+  // Instances with the most rows first (their tiles take longest), each
+  // instance's tiles together; std::sort works in place.
+  for (uint32_t k = 0; k < count; ++k) g_order[k] = k;
+  std::sort(g_order, g_order + count, [&](uint32_t a, uint32_t b) {
+    return iterations[a] != iterations[b] ? iterations[a] > iterations[b] : a < b;
+  });
+  rngi::NoallocArgs args;
+  const bool few = count <= rngi::kNoallocFew;
+  rngi::BatchInstance *inst = few ? args.few : g_host.inst;
+  uint32_t *first = few ? args.few_first : g_host.first;
+  uint32_t tiles = 0;
+  for (uint32_t i = 0; i < count; ++i) {
+    const uint32_t k = g_order[i];
+    rngi::BatchInstance &in = inst[i];
     in.out = outs[k];
     in.state = nullptr;
     in.streams = streams[k];
@@ -104,28 +112,24 @@ extern "C" int rng_batch_generate_noalloc(uint32_t count, const uint64_t *stream
     in.vec = (streams[k] % 2 == 0) && (reinterpret_cast<uintptr_t>(outs[k]) % 16 == 0);
     in.from_hash = 1;
     in.write_state = 0;
-    for (uint64_t s = 0; s < streams[k]; s += kTile)
-      g_host_units[u++] = {k, static_cast<uint32_t>(std::min(kTile, streams[k] - s)), s};
+    first[i] = tiles;
+    tiles += static_cast<uint32_t>((streams[k] + kTile - 1) / kTile);
   }
-  // Largest units first; ties in table order (std::sort works in place).
-  std::sort(g_host_units, g_host_units + u, [](const rngi::BatchUnit &a, const rngi::BatchUnit &b) {
-    const uint64_t wa = uint64_t(a.count) * g_host_inst[a.inst].rows;
-    const uint64_t wb = uint64_t(b.count) * g_host_inst[b.inst].rows;
-    if (wa != wb) return wa > wb;
-    if (a.inst != b.inst) return a.inst < b.inst;
-    return a.s_begin < b.s_begin;
-  });
+  args.count = count;
+  args.inst = nullptr;
+  args.first = nullptr;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // From pageable memory these copies return once the source has been read,
-  // so the staging arrays can be refilled by the next call.
-  st = cudaMemcpyAsync(d_inst, g_host_inst, count * sizeof(rngi::BatchInstance), cudaMemcpyHostToDevice, s);
-  if (st == cudaSuccess)
-    st = cudaMemcpyAsync(d_units, g_host_units, u * sizeof(rngi::BatchUnit), cudaMemcpyHostToDevice, s);
-  if (st == cudaSuccess) st = cudaMemsetAsync(d_counter, 0, sizeof(uint32_t), s);  // must start at zero
-  if (st != cudaSuccess) return rngi::cuda_fail(err, st, "rng_batch_generate_noalloc: table upload");
-  const int per_sm = rngi::batch_blocks_per_sm(kVpt, kBlock);
-  const uint64_t resident = uint64_t(rngi::device_sm_count(dev)) * (per_sm > 0 ? per_sm : 1);
-  const uint32_t grid = static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(resident, u)));
-  st = rngi::launch_batch(d_inst, d_units, u, d_counter, kVpt, kBlock, grid, s);
+  if (!few) {
+    // From pageable memory these copies return once the source has been read,
+    // so the staging arrays can be refilled by the next call.
+    unsigned char *base = g_scratch_addr[dev];
+    st = cudaMemcpyAsync(base, g_host.inst, count * sizeof(rngi::BatchInstance), cudaMemcpyHostToDevice, s);
+    if (st == cudaSuccess)
+      st = cudaMemcpyAsync(base + kInstBytes, g_host.first, count * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
+    if (st != cudaSuccess) return rngi::cuda_fail(err, st, "rng_batch_generate_noalloc: table upload");
+    args.inst = reinterpret_cast<const rngi::BatchInstance *>(base);
+    args.first = reinterpret_cast<const uint32_t *>(base + kInstBytes);
+  }
+  st = rngi::launch_noalloc(args, tiles, s);
   return rngi::cuda_fail(err, st, "rng_batch_generate_noalloc: kernel launch");
 }
