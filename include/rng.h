@@ -315,6 +315,12 @@ int rng_set_state(rng_gen *g, const uint64_t *host_states, uint64_t position, rn
 int rng_sync(rng_gen *g, rng_err **err);
 /* The compute stream (cudaStream_t) the generator launches on. */
 void *rng_compute_stream(rng_gen *g);
+/* Order the generator's work with a stream of the caller's (a cudaStream_t of
+ * the same device), by an event: what the generator launches next starts
+ * after what `stream` has queued (rng_follow_stream); what `stream` is given
+ * next starts after what the generator has queued (rng_lead_stream). */
+int rng_follow_stream(rng_gen *g, void *stream, rng_err **err);
+int rng_lead_stream(rng_gen *g, void *stream, rng_err **err);
 /* Register-store launch configuration chosen for `streams` at creation:
  * values per thread, threads per block and blocks of the grid.  A device
  * output may run the bulk-copy row kernel in another shape instead (see

@@ -131,6 +131,8 @@ SIGNATURES = {
     "rng_get_state": ([c_vp, c_vp, P_err], c_int),
     "rng_set_state": ([c_vp, c_vp, c_u64, P_err], c_int),
     "rng_sync": ([c_vp, P_err], c_int),
+    "rng_follow_stream": ([c_vp, c_vp, P_err], c_int),
+    "rng_lead_stream": ([c_vp, c_vp, P_err], c_int),
     "rng_compute_stream": ([c_vp], c_vp),
     "rng_launch_config": ([c_vp, ctypes.POINTER(c_u32), ctypes.POINTER(c_u32), ctypes.POINTER(c_u32)], c_int),
     "rng_last_launch": ([c_vp, ctypes.POINTER(RngLaunchInfo), P_err], c_int),

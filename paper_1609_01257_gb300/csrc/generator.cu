@@ -73,6 +73,7 @@ struct rng_gen {
   std::vector<void *> h_slots;
   std::vector<void *> h_slots_dev;  // the slots' device-side addresses
   std::vector<cudaEvent_t> slot_ready;
+  cudaEvent_t order = nullptr;      // rng_follow_stream, rng_lead_stream
   cudaEvent_t produced[2] = {nullptr, nullptr}, copied[2] = {nullptr, nullptr};
   // profiling
   std::vector<cudaEvent_t> evpool;
@@ -783,6 +784,7 @@ int rng_create(uint64_t streams, uint64_t seed, const rng_opts *opts, rng_gen **
   }
   if (!rc) rc = rngi::cuda_fail(err, cudaStreamCreateWithFlags(&g->copy, cudaStreamNonBlocking), "cudaStreamCreate");
   if (!rc) rc = rngi::cuda_fail(err, cudaMalloc(&g->d_state, streams * 8), "cudaMalloc(state)");
+  if (!rc) rc = rngi::cuda_fail(err, cudaEventCreateWithFlags(&g->order, cudaEventDisableTiming), "cudaEventCreate");
   if (!rc) rc = profile_restart(g, err);
   if (!rc) g->prof = rngi::prof_create_owned();
   if (!rc && !g->prof) rc = rngi::fail(err, RNG_ENOMEM, "rng_create: profiler allocation failed");
@@ -812,6 +814,7 @@ void rng_destroy(rng_gen *g) {
   for (cudaEvent_t e : g->slot_ready) cudaEventDestroy(e);
   for (cudaEvent_t e : g->evpool) cudaEventDestroy(e);
   if (g->origin) cudaEventDestroy(g->origin);
+  if (g->order) cudaEventDestroy(g->order);
   if (g->copy) cudaStreamDestroy(g->copy);
   if (g->own_compute && g->compute) cudaStreamDestroy(g->compute);
   rngi::prof_destroy_owned(g->prof);
@@ -1129,6 +1132,25 @@ int rng_sync(rng_gen *g, rng_err **err) {
 }
 
 void *rng_compute_stream(rng_gen *g) { return g ? static_cast<void *>(g->compute) : nullptr; }
+
+// One event for both: a wait takes the event's last record at the time of the
+// call, so it can be recorded again at once.
+static int order_streams(rng_gen *g, cudaStream_t first, cudaStream_t then, const char *fn, rng_err **err) {
+  if (first == then) return RNG_OK;
+  cudaError_t st = cudaEventRecord(g->order, first);
+  if (st == cudaSuccess) st = cudaStreamWaitEvent(then, g->order, 0);
+  return rngi::cuda_fail(err, st, fn);
+}
+
+int rng_follow_stream(rng_gen *g, void *stream, rng_err **err) {
+  const int rc = check_gen(g, err, "rng_follow_stream");
+  return rc ? rc : order_streams(g, static_cast<cudaStream_t>(stream), g->compute, "rng_follow_stream", err);
+}
+
+int rng_lead_stream(rng_gen *g, void *stream, rng_err **err) {
+  const int rc = check_gen(g, err, "rng_lead_stream");
+  return rc ? rc : order_streams(g, g->compute, static_cast<cudaStream_t>(stream), "rng_lead_stream", err);
+}
 
 int rng_launch_config(const rng_gen *g, uint32_t *vpt, uint32_t *block, uint32_t *grid) {
   if (!g) return RNG_EINVAL;

@@ -13,6 +13,9 @@
 // xorshift), so every output equals the same request served alone.
 #include <cuda_runtime.h>
 #include <string.h>
+#ifdef __linux__
+#include <sys/prctl.h>
+#endif
 
 #include <algorithm>
 #include <chrono>
@@ -290,6 +293,11 @@ struct rng_server {
 
   void run() {
     cudaSetDevice(device);
+#ifdef __linux__
+    // This thread's short sleeps end when they should: with the default slack
+    // of 50 us the 20 us polls below take about 75.
+    prctl(PR_SET_TIMERSLACK, 1000UL, 0UL, 0UL, 0UL);
+#endif
     std::unique_lock<std::mutex> lk(mu);
     for (;;) {
       complete_steps_locked();

@@ -134,32 +134,35 @@ class Generator:
                 "values_per_thread": info.values_per_thread, "block": info.block_threads,
                 "grid": info.grid_blocks, "row_buffers": info.row_buffers, "band_rows": info.band_rows}
 
-    def _after_current(self):
+    def _after_current(self) -> int:
         # The library's work follows what torch's current stream has queued
         # (e.g. the output's allocation) ...
-        ev = torch.cuda.Event()
-        ev.record(torch.cuda.current_stream(self.device))
-        self.stream.wait_event(ev)
+        current = torch.cuda.current_stream(self.device).cuda_stream
+        C.check(self._lib.rng_follow_stream, self._h, current)
+        return current
 
-    def _before_current(self):
+    def _before_current(self, current: int):
         # ... and torch's current stream waits for it, so that a tensor handed
         # back is ready for whatever the caller queues next (``.cpu()``, ...).
-        ev = torch.cuda.Event()
-        ev.record(self.stream)
-        torch.cuda.current_stream(self.device).wait_event(ev)
+        C.check(self._lib.rng_lead_stream, self._h, current)
 
     def generate(self, iterations: int, out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """Next ``iterations`` rows on the device.  Asynchronous for the host:
         the kernel runs on the generator's compute stream, and torch's current
         stream is made to wait for it before the tensor is returned."""
-        if out is None:
+        fresh = out is None
+        if fresh:
             out = torch.empty((iterations, self.streams), dtype=torch.uint64, device=self.device)
-        assert out.is_cuda and out.is_contiguous() and out.element_size() == 8
-        assert out.numel() >= iterations * self.streams
-        self._after_current()
-        C.check(self._lib.rng_generate, self._h, iterations, ctypes.c_void_p(out.data_ptr()), None)
-        out.record_stream(self.stream)
-        self._before_current()
+        else:
+            assert out.is_cuda and out.is_contiguous() and out.element_size() == 8
+            assert out.numel() >= iterations * self.streams
+        current = self._after_current()
+        C.check(self._lib.rng_generate, self._h, iterations, out.data_ptr(), None)
+        if not fresh:
+            # Its memory may belong to any stream; memory allocated here is the
+            # current stream's, which waits for the kernel below.
+            out.record_stream(self.stream)
+        self._before_current(current)
         return out
 
     def generate_to(self, iterations: int, out_ptr: int):
@@ -171,11 +174,11 @@ class Generator:
         tensor), row ``i mod R`` for iteration ``i``; asynchronous."""
         assert ring.is_cuda and ring.is_contiguous() and ring.element_size() == 8
         assert ring.numel() % self.streams == 0 and ring.numel() >= self.streams
-        self._after_current()
+        current = self._after_current()
         C.check(self._lib.rng_generate_ring, self._h, iterations, ctypes.c_void_p(ring.data_ptr()),
                 ring.numel() // self.streams)
         ring.record_stream(self.stream)
-        self._before_current()
+        self._before_current(current)
         return ring
 
     def generate_to_host(self, iterations: int, out=None):
@@ -255,12 +258,12 @@ class Generator:
             row_xor = torch.empty(iterations, dtype=torch.uint64, device=self.device)
         if row_sum is None:
             row_sum = torch.empty(iterations, dtype=torch.uint64, device=self.device)
-        self._after_current()
+        current = self._after_current()
         C.check(self._lib.rng_generate_checksum, self._h, iterations,
                 ctypes.c_void_p(row_xor.data_ptr()), ctypes.c_void_p(row_sum.data_ptr()))
         row_xor.record_stream(self.stream)
         row_sum.record_stream(self.stream)
-        self._before_current()
+        self._before_current(current)
         return row_xor, row_sum
 
     def state(self) -> np.ndarray:
