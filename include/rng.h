@@ -94,9 +94,9 @@ typedef struct rng_opts {
     int32_t device;               /* CUDA device ordinal; -1 = current device */
     uint32_t store_policy;        /* 0 = default stores, 1 (default) = streaming
                                      stores (st.global.cs, evict-first), with
-                                     the bulk-copy kernel where it measured
-                                     faster (device outputs of at least 128
-                                     rows per call) when the shape is left to
+                                     the bulk-copy kernels where they measured
+                                     faster (device outputs of many rows per
+                                     call) when the shape is left to
                                      the library (values_per_thread,
                                      block_threads, grid_blocks and
                                      store_width all 0); 2 =
@@ -294,8 +294,9 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
 /* Jump-ahead: advances every stream by `iterations` iterations without
  * producing them (position p += iterations, modulo 2^64).  The update of
  * Listing S5 is linear over GF(2), so k iterations are one multiplication by
- * the k-th power of its 64x64 bit matrix, computed on the host by repeated
- * squaring and applied by one kernel (64 conditional XORs per stream).  The
+ * the k-th power of its 64x64 bit matrix, computed on the host from x^k modulo
+ * the matrix's characteristic polynomial and applied by one kernel (table
+ * lookups).  The
  * update has period 2^64 - 1: skipping that many returns every stream to its
  * current state.  For resuming a run, checkpoints, and splitting a run by
  * iterations across callers.  Ordered on the compute stream. */

@@ -223,10 +223,16 @@ int gen_launch_rows(rng_gen *g, rngi::RowsLaunch &a, const rngi::LaunchShape &sh
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool may_band = !a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n &&
                         cudaStreamIsCapturing(g->compute, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  const rngi::LaunchShape sh = rngi::resolve_shape(base, a, may_band);
+  rngi::LaunchShape sh = rngi::resolve_shape(base, a, may_band);
   bool swap = false;
   if (may_band) {
-    const uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
+    uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
+    if (br && band_memory(g, static_cast<uint32_t>(std::min<uint64_t>((a.rows + br - 1) / br, rngi::kMaxBands)),
+                          !a.from_hash) != cudaSuccess) {
+      // No memory for bands: slower without them, but not an error.
+      sh = rngi::resolve_shape(base, a, false);
+      br = 0;
+    }
     if (br) {
       int rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
       if (rc) return rc;
@@ -994,8 +1000,9 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   if (iterations == 0) return RNG_OK;
   rc = size_ok(g->n, iterations, err);
   if (rc) return rc;
-  cudaError_t st = rngi::launch_zero_pair(row_xor_dev, row_sum_dev, iterations, g->compute);
-  rc = rngi::cuda_fail(err, st, "checksum reset launch");
+  cudaError_t st = cudaMemsetAsync(row_xor_dev, 0, iterations * 8, g->compute);
+  if (st == cudaSuccess) st = cudaMemsetAsync(row_sum_dev, 0, iterations * 8, g->compute);
+  rc = rngi::cuda_fail(err, st, "cudaMemsetAsync(checksums)");
   if (rc) return rc;
   rngi::RowsLaunch a{};
   a.state = g->d_state;

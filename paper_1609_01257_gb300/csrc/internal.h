@@ -51,7 +51,6 @@ const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb);
 const void *noalloc_kernel_fn();
 const void *init_kernel_fn();
 const void *copy_kernel_fn();
-const void *zero_pair_kernel_fn();
 
 // Sets *err (when err != NULL and *err == NULL) and returns `code`.
 int fail(rng_err **err, int code, const char *fmt, ...) __attribute__((format(printf, 3, 4)));
@@ -158,8 +157,6 @@ cudaError_t launch_jump(uint64_t *state, uint64_t n, uint64_t id_base, uint32_t 
 // Values per thread of a generate-and-checksum launch of `rows` rows over
 // `span` streams (vpt = 0: choose; else a power of two up to 64).
 uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt);
-// x[0 .. n-1] = s[0 .. n-1] = 0 in one launch.
-cudaError_t launch_zero_pair(uint64_t *x, uint64_t *s, uint64_t n, cudaStream_t st);
 // Generate-and-checksum launch with `vpt` values per thread; a.band_rows != 0
 // selects the banded variant (a.jump, a.state_out as for the row kernel).
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,

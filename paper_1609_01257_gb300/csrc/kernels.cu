@@ -10,8 +10,13 @@
 // Nothing is read per value; the state array is touched once at the start
 // and once at the end.
 //
+// Launches of many rows stage each row in shared memory and write it by TMA
+// bulk copies instead, paced under the rate that HBM takes.
+//
 // Also here: the generate-and-checksum kernel, the work-list kernels of the
-// batched, served and allocation-free forms, the init kernel, and the copy kernel of the double buffer's copy-kernel reads.
+// batched, served and allocation-free forms, the init kernel, and the copy
+// kernel of the double buffer's copy-kernel reads.  The bit-sliced checksum
+// kernel is in checksum_sliced.cu, the jump-ahead in jump.cu.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -521,15 +526,6 @@ __global__ void init_kernel(uint64_t *__restrict__ state, uint64_t n, uint64_t i
   for (uint64_t s = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; s < n;
        s += static_cast<uint64_t>(gridDim.x) * blockDim.x)
     state[s] = prng::initial_state(id_base + s, key);
-}
-
-// Clears two arrays of n words.
-__global__ void zero_pair_kernel(uint64_t *x, uint64_t *s, uint64_t n) {
-  for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-    x[i] = 0;
-    s[i] = 0;
-  }
 }
 
 // Device-to-host read of one double-buffer chunk done by SMs instead of the
@@ -1102,7 +1098,6 @@ const void *batch_work_bulk_kernel_fn(uint32_t vpt, uint32_t nb) {
 }
 const void *noalloc_kernel_fn() { return reinterpret_cast<const void *>(&noalloc_kernel<kNoallocVpt>); }
 const void *init_kernel_fn() { return reinterpret_cast<const void *>(&init_kernel); }
-const void *zero_pair_kernel_fn() { return reinterpret_cast<const void *>(&zero_pair_kernel); }
 const void *copy_kernel_fn() { return reinterpret_cast<const void *>(&copy_kernel); }
 
 }  // namespace rngi

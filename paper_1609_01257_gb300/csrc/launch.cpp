@@ -377,14 +377,17 @@ cudaError_t launch_copy(uint64_t *dst, const uint64_t *src, uint64_t n, cudaStre
   return e;
 }
 
-// Row kernel (bound by HBM writes): bands only when the tiles cannot cover
-// half the SMs (128 unbanded tiles of 2^16 streams ran at 7.37 TB/s, three
-// bands of them at 6.25); then about two (tile, band) units per SM (16 tiles
-// of 4096 streams: 19 bands 6.6 TB/s, 10 bands 4.7 TB/s).
+// Register and staged row kernels (bound by HBM writes): bands only when the
+// tiles cannot cover half the SMs (128 unbanded tiles of 2^16 streams ran at
+// 7.37 TB/s, three bands of them at 6.25: more SMs than HBM takes writes
+// from, see Pacer in kernels.cu); then about two (tile, band) units per SM
+// (16 tiles of 4096 streams: 19 bands 6.6 TB/s, 10 bands 4.7 TB/s).  A bulk
+// plan carries its own bands.
 // Checksum kernel (bound by integer issue): bands whenever the tiles leave
 // resident block slots empty, up to about four units per slot, so that the
 // last wave of units is a small part of the launch.
-// Bands hold at least 128 rows, which amortises each unit's jump.
+// Bands hold at least 128 rows (64 in the checksum kernel), which amortises
+// each unit's jump.
 uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh, int device, bool checksum,
                           uint32_t out) {
   const uint64_t sms = static_cast<uint64_t>(device_sm_count(device));
@@ -452,14 +455,6 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
     v /= 2;
   }
   return v;
-}
-
-cudaError_t launch_zero_pair(uint64_t *x, uint64_t *s, uint64_t n, cudaStream_t st) {
-  const uint64_t blocks = std::min<uint64_t>((n + 255) / 256, 1024);
-  void *params[] = {&x, &s, &n};
-  const cudaError_t e = cudaLaunchKernel(zero_pair_kernel_fn(), dim3(static_cast<unsigned>(blocks)), dim3(256), params, 0, st);
-  if (e == cudaSuccess) count_launch();
-  return e;
 }
 
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,
