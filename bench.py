@@ -54,11 +54,10 @@ WORKLOADS = {
                   name="plain method: 2^16 streams x 100 iterations, seed 0"),
 }
 
-# ALU-pipe lane operations per value of checksum_kernel<16> in output modes
-# 0 and 1, from their ncu captures: ALU-pipe utilisation (85.5 %, 74.9 %) x 64
-# lanes x 152 SMs x 1.85 GHz x duration (184.2 us, 209.7 us) over 2^22 x 64
-# values.
-CHECKSUM_ALU_OPS_PER_VALUE = {0: 10.6, 1: 10.5}
+# ALU-pipe lane operations per value of the generate-and-checksum kernels on
+# large launches in output modes 0 (bit-sliced) and 1, from their ncu captures:
+# ALU-pipe warp instructions x 32 / values over 2^22 streams x 512 and 64 rows.
+CHECKSUM_ALU_OPS_PER_VALUE = {0: 5.95, 1: 9.43}
 NOMINAL_HBM_GBPS = 7900.0  # GB300 HBM3e, nominal
 METRIC = "GB/s of uint64 PRNG output (device and host-streamed) vs roofline; p50/p99 req latency"
 
