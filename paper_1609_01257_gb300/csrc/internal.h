@@ -32,6 +32,8 @@ const void *rows_staged_kernel_fn(uint32_t vpt, bool banded, uint32_t out);
 // 4; 256-thread blocks), and its dynamic shared memory in bytes.
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out);
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb);
+// Rings of more rows than this do not hold the bulk-copy row kernel up.
+constexpr int kBulkRingRows = 32;
 // Banded row kernel of few streams (at most 256 * vpt; vpt 1, 2, 4, 8 or 16):
 // several rows per bulk copy.
 const void *rows_multi_kernel_fn(uint32_t vpt, uint32_t out);

@@ -207,8 +207,30 @@ template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
-// Waits until all of this thread's groups are complete (their writes done).
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// Waits until at most N of this thread's committed groups are incomplete (the
+// others' writes are done).
+template <int N>
+__device__ __forceinline__ void bulk_wait() {
+  asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { bulk_wait<0>(); }
+
+// Before the copy of a row goes to an address of a ring of `ring` rows: waits
+// until the copy of the row before it there, `ring` copies back, is complete.
+// Bulk copies have no order among themselves, and the wait for a buffer
+// covers only its reads.  At most ring - 1 copies may be open, one of three
+// counts; 32 rows back a copy has long been done, so larger rings do not wait
+// (GB300, 2^20 streams x 512 rows, 8 values per thread: rings of up to 10 rows
+// 786 us, of up to 32 663, larger ones 643).
+template <int NB>
+__device__ __forceinline__ void bulk_wait_ring(uint64_t ring) {
+  if (ring > kBulkRingRows)
+    bulk_wait<kBulkRingRows>();
+  else if (ring > NB - 2)
+    bulk_wait<NB - 2>();
+  else
+    bulk_wait<0>();
+}
 
 // Issue times of a block's bulk copies.  One SM can write 32 bytes a clock
 // (62 GB/s), so from about 130 of the 152 SMs on they offer more than HBM
@@ -260,8 +282,8 @@ __host__ __device__ constexpr int bulk_words() {
 // SMs' store path then carries only shared-memory writes.  A buffer is
 // refilled only after the copy that read it NB rows earlier has finished
 // reading.  Values past `span` are staged but not copied.  ring != 0: rows
-// wrap around a ring of `ring` rows.  Every thread of the block must call
-// it; the issuing thread must wait for its groups (bulk_wait_all) before the
+// wrap around a ring of `ring` rows, and a row's copy waits for the one before
+// it at its place.  Every thread of the block must call it; the issuing thread must wait for its groups (bulk_wait_all) before the
 // block exits.
 template <int VPT, int NB, int OUT = 0>
 __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *row, uint64_t pitch, uint64_t rows,
@@ -288,6 +310,7 @@ __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *ro
       // copy issued NB - 1 rows before this one: at most NB - 2 later copies
       // may still be reading.
       if (warm + 1 >= NB) bulk_wait_read<NB - 2>();
+      if (ring && r >= ring) bulk_wait_ring<NB>(ring);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
