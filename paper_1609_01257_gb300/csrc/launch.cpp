@@ -104,7 +104,7 @@ uint32_t ceil16(uint64_t v) { return static_cast<uint32_t>((v + 15) / 16 * 16); 
 // The bulk-copy kernels for one launch of `rows` rows over `streams` streams
 // when the caller leaves the shape to the library, for rows on 128-byte lines
 // (`lined`) and off them; nb == 0: keep the register or staged kernels.
-// may_band: the rows may be split into bands; out_bytes: the output's size
+// may_band: the rows may be split into bands; out_rows: rows of the output
 // (the ring's, when rows wrap).  One block per SM, all with equal shares:
 // tiles and bands come to whole rounds of the SMs, because a paced block does
 // not use what another leaves (1000003 streams x 512 rows, 16 values per
@@ -122,11 +122,17 @@ uint32_t ceil16(uint64_t v) { return static_cast<uint32_t>((v + 15) / 16 * 16); 
 //    + 1 x 64 317 / 306; at 16 rows even or worse;
 //  - on the lines, 2^20 x 255 307 / 292, 2^22 x 128 602 / 584, 65536 x 4096 293 /
 //    294 (and 340 where 128 unpaced SMs are past the ceiling); 2^22 x 64 308 /
-//    324, 2^24 x 32 656 / 690 (each tile's loads are exposed).
-BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, uint64_t out_bytes, uint32_t sms) {
+//    324, 2^24 x 32 656 / 690 (each tile's loads are exposed);
+//  - rings on the lines: what a small one overwrites stays in the L2, 2^20 x
+//    512 into 16 or 64 rows 489 or 550 / 580, into 128 (1 GB) 611 / 581;
+//  - without bands, fewer tiles than half the SMs would be cut into pieces of a
+//    few KB, each of which takes its block the 0.4 us: rings of 65536 x 8192
+//    553 / 3400, 70001 x 300 41 / 146.
+BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, uint64_t out_rows, uint32_t sms) {
   constexpr uint64_t M = uint64_t(1) << 20;
   BulkPlan p;
-  const uint64_t bytes = 8 * streams * rows;
+  const bool ring = out_rows < rows;
+  const uint64_t bytes = 8 * streams * out_rows;
   uint64_t units;
   if (streams <= 4096) {
     if (!may_band || rows < (lined ? 16 * uint64_t(sms) : 64)) return p;
@@ -146,8 +152,9 @@ BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, u
     p.nb = bulk_buffers(p.vpt);
     const uint64_t most = uint64_t(kGenBlock) * p.vpt;
     const uint64_t tiles = (streams + most - 1) / most;
+    if (!may_band && tiles * 2 <= sms) return BulkPlan{};
     if (lined) {
-      if (many ? rows < 128 : rows <= 128 || bytes < (tiles < sms ? 1024 : 256) * M) return BulkPlan{};
+      if (many ? rows < 128 : rows <= 128 || bytes < (ring || tiles < sms ? 1024 : 256) * M) return BulkPlan{};
     } else if (rows < (streams < uint64_t(sms) * 1024 ? 128 : many ? 16 : 32)) {
       return BulkPlan{};
     }
@@ -175,7 +182,7 @@ BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, u
   }
   p.blocks = static_cast<uint32_t>(std::min<uint64_t>(units, sms));
   // Outputs that the 129 MB L2 can take are written as fast as it takes them.
-  if (out_bytes >= 128 * M) p.pace = pace_of(p.blocks);
+  if (bytes >= 128 * M) p.pace = pace_of(p.blocks);
   return p;
 }
 
@@ -256,8 +263,7 @@ LaunchShape resolve_shape(const LaunchShape &sh, const RowsLaunch &a, bool may_b
     r.bulk.nb = bulk_buffers(sh.vpt);
     r.bulk.tile_w = kGenBlock * sh.vpt;
   } else if (sh.bulk_auto) {
-    r.bulk = bulk_plan(span, a.rows, lined, may_band,
-                       8 * span * (a.ring_rows && a.ring_rows < a.rows ? a.ring_rows : a.rows), sh.sms);
+    r.bulk = bulk_plan(span, a.rows, lined, may_band, a.ring_rows ? std::min(a.ring_rows, a.rows) : a.rows, sh.sms);
   }
   if (!r.bulk.nb) {
     const uint32_t v = sh.bulk_auto && !lined ? direct_vpt(span) : 0;
