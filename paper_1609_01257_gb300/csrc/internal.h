@@ -31,6 +31,7 @@ const void *rows_staged_kernel_fn(uint32_t vpt, bool banded, uint32_t out);
 // buffers (4 values per thread with 8 buffers, 8 with 12, 16 with 6, 24 with
 // 4; 256-thread blocks), and its dynamic shared memory in bytes.
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out);
+const void *rows_bulk_ring_kernel_fn(uint32_t vpt, uint32_t nb, uint32_t out);  // rows wrap; vpt 4, 8 or 16
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb);
 // Rings of more rows than this do not hold the bulk-copy row kernel up.
 constexpr int kBulkRingRows = 32;

@@ -241,6 +241,7 @@ __device__ __forceinline__ void bulk_wait_ring(uint64_t ring) {
 // SM every 316-324 ns wrote 7.65-7.79 TB/s in a copy-only kernel (memset
 // 7.58), 310 ns 7.1-7.3, unpaced 6.66.
 struct Pacer {
+  uint32_t rate;     // 2^-20 ns per byte
   uint64_t t0 = 0;   // when the schedule began (ns)
   uint64_t due = 0;  // since then (2^-20 ns)
   // The time, to be read before the block's barrier so that its latency is
@@ -250,18 +251,24 @@ struct Pacer {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
   }
-  // Waits for the turn of copies of `bytes`, `t` being a reading of now();
-  // rate: 2^-20 ns per byte, 0 = no schedule.  A block that is late by more
-  // than a microsecond (a new tile's states were loaded) goes on from there
-  // instead of catching up in a burst.
-  __device__ __forceinline__ void wait(uint64_t t, uint32_t bytes, uint32_t rate) {
-    if (!rate) return;
+  // Waits for the turn of copies of `bytes`, `t` being a reading of now().  A
+  // block that is late by more than a microsecond (a new tile's states were
+  // loaded) goes on from there instead of catching up in a burst.
+  __device__ __forceinline__ void wait(uint64_t t, uint32_t bytes) {
     if (!t0) t0 = t;
     const uint64_t turn = t0 + (due >> 20);
     for (int polls = 0; polls < 4096 && t < turn; ++polls) t = now();
     if (t > turn + 1024) t0 += t - turn - 1024;
     due += static_cast<uint64_t>(bytes) * rate;
   }
+};
+
+// Copies without a schedule: a type of its own, since a rate of 0 that is
+// looked at in every row made short rows 10 to 37 % slower (65536 streams x
+// 130 rows, 4 values per thread: 31 us, 41 with the test).
+struct Unpaced {
+  static __device__ __forceinline__ uint64_t now() { return 0; }
+  __device__ __forceinline__ void wait(uint64_t, uint32_t) {}
 };
 
 // Shared words of the bulk row kernel: NB row buffers of one tile plus two
@@ -281,14 +288,14 @@ __host__ __device__ constexpr int bulk_words() {
 // 8-byte stores of an odd head or tail, at the time the pacer gives.  The
 // SMs' store path then carries only shared-memory writes.  A buffer is
 // refilled only after the copy that read it NB rows earlier has finished
-// reading.  Values past `span` are staged but not copied.  ring != 0: rows
-// wrap around a ring of `ring` rows, and a row's copy waits for the one before
-// it at its place.  Every thread of the block must call it; the issuing thread must wait for its groups (bulk_wait_all) before the
+// reading.  Values past `span` are staged but not copied.  RING: rows wrap
+// around a ring of `ring` rows, and a row's copy waits for the one before it at
+// its place.  Every thread of the block must call it; the issuing thread must wait for its groups (bulk_wait_all) before the
 // block exits.
-template <int VPT, int NB, int OUT = 0>
+template <int VPT, int NB, int OUT = 0, bool RING = false, class Pace>
 __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *row, uint64_t pitch, uint64_t rows,
                                                uint64_t span, uint64_t ring, uint64_t *buf, uint32_t &kb,
-                                               uint32_t &warm, Pacer &pacer, uint32_t pace) {
+                                               uint32_t &warm, Pace &pacer) {
   static_assert(NB >= 2, "NB: at least 2");
   constexpr int kTile = kBlock * VPT;
   constexpr int kBuf = kTile + 2;
@@ -305,17 +312,17 @@ __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *ro
     fence_proxy_async_smem();
     uint64_t t = 0;
     if (threadIdx.x == 0) {
-      if (pace) t = Pacer::now();
+      t = Pace::now();
       // After this barrier the block fills the next buffer, last read by the
       // copy issued NB - 1 rows before this one: at most NB - 2 later copies
       // may still be reading.
       if (warm + 1 >= NB) bulk_wait_read<NB - 2>();
-      if (ring && r >= ring) bulk_wait_ring<NB>(ring);
+      if (RING && r >= ring) bulk_wait_ring<NB>(ring);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       const int body = (n - p) & ~1;
-      pacer.wait(t, 8u * static_cast<uint32_t>(n), pace);
+      pacer.wait(t, 8u * static_cast<uint32_t>(n));
       if (p) store_one<kPolicyStreaming>(row, b[1]);
       if ((n - p) & 1) store_one<kPolicyStreaming>(row + n - 1, b[p + n - 1]);
       if (body > 0) bulk_store(row + p, b + 2 * p, 8u * static_cast<uint32_t>(body));
@@ -324,7 +331,7 @@ __device__ __forceinline__ void emit_rows_bulk(uint64_t (&st)[VPT], uint64_t *ro
     kb = kb + 1 == NB ? 0 : kb + 1;
     if (warm < NB) ++warm;
     row += pitch;
-    if (ring && ++in_ring == ring) {
+    if (RING && ++in_ring == ring) {
       row = first;
       in_ring = 0;
     }
@@ -436,21 +443,20 @@ __global__ void __launch_bounds__(kBlock) rows_staged_kernel(const RowsLaunch a)
 
 // Row kernel whose rows are written by TMA bulk copies from shared memory
 // (emit_rows_bulk): work units as in rows_staged_kernel but for the tile's
-// width, any row alignment, and rings when unbanded.  A tile is a.tile_w <=
+// width, any row alignment, and rings in a variant of their own (their waits
+// cost the row loop of other launches 10 %).  A tile is a.tile_w <=
 // kBlock * VPT streams, chosen by the host so that the tiles come to whole
 // waves of the SMs (see bulk_plan); the threads' values past it are computed
 // and staged, not copied, which costs nothing here (the row loop waits for
 // HBM).  The dynamic shared memory holds the NB row buffers
 // (bulk_words<VPT, NB>() words).
-template <int VPT, int NB, bool BANDED, int OUT = 0>
-__global__ void __launch_bounds__(kBlock) rows_bulk_kernel(const RowsLaunch a) {
-  extern __shared__ __align__(128) uint64_t bulk_buf[];
+template <int VPT, int NB, bool BANDED, int OUT, bool RING, class Pace>
+__device__ __forceinline__ void rows_bulk_units(const RowsLaunch &a, uint64_t *buf, Pace pacer) {
   const uint64_t span = a.s_end - a.s_begin;
   const uint64_t n_tiles = (span + a.tile_w - 1) / a.tile_w;
   const uint64_t band_rows = BANDED ? a.band_rows : a.rows;
   const uint64_t n_bands = BANDED ? (a.rows + band_rows - 1) / band_rows : 1;
   uint32_t kb = 0, warm = 0;
-  Pacer pacer;
   for (uint64_t w = blockIdx.x; w < n_tiles * n_bands; w += gridDim.x) {
     const uint64_t tile = w % n_tiles;
     const uint64_t band = BANDED ? w / n_tiles : 0;
@@ -464,12 +470,25 @@ __global__ void __launch_bounds__(kBlock) rows_bulk_kernel(const RowsLaunch a) {
     }
     const uint64_t r0 = band * band_rows;
     const uint64_t rows = BANDED ? (a.rows - r0 < band_rows ? a.rows - r0 : band_rows) : a.rows;
-    emit_rows_bulk<VPT, NB, OUT>(st, a.out + r0 * a.pitch + rel0, a.pitch, rows, end - rel0,
-                                 BANDED ? 0 : a.ring_rows, bulk_buf, kb, warm, pacer, a.pace);
+    emit_rows_bulk<VPT, NB, OUT, RING>(st, a.out + r0 * a.pitch + rel0, a.pitch, rows, end - rel0, a.ring_rows, buf, kb,
+                                       warm, pacer);
     if (a.write_state && band == n_bands - 1)
       store_tile_state<VPT, 1>(st, BANDED ? a.state_out : a.state, a, rel0, end);
   }
   if (threadIdx.x == 0) bulk_wait_all();
+}
+
+// Plans pace launches of 16 and 24 values per thread only (bulk_plan).
+template <int VPT, int NB, bool BANDED, int OUT = 0, bool RING = false>
+__global__ void __launch_bounds__(kBlock) rows_bulk_kernel(const RowsLaunch a) {
+  extern __shared__ __align__(128) uint64_t bulk_buf[];
+  if constexpr (VPT >= 16) {
+    if (a.pace) {
+      rows_bulk_units<VPT, NB, BANDED, OUT, RING>(a, bulk_buf, Pacer{a.pace});
+      return;
+    }
+  }
+  rows_bulk_units<VPT, NB, BANDED, OUT, RING>(a, bulk_buf, Unpaced{});
 }
 
 // Few streams (at most kBlock * VPT, the whole row in every block) and many
@@ -496,7 +515,7 @@ __global__ void __launch_bounds__(kBlock) rows_multi_kernel(const RowsLaunch a) 
 #pragma unroll
   for (int j = 0; j < VPT; ++j) in[j] = static_cast<int>(threadIdx.x) + kBlock * j < n;
   uint32_t kb = 0, warm = 0;
-  Pacer pacer;
+  Pacer pacer{a.pace};
   for (uint64_t band = blockIdx.x; band < n_bands; band += gridDim.x) {
     uint64_t st[VPT];
     load_tile<VPT, 1>(st, a, 0, span);
@@ -528,7 +547,7 @@ __global__ void __launch_bounds__(kBlock) rows_multi_kernel(const RowsLaunch a) 
       __syncthreads();
       if (threadIdx.x == 0) {
         const int count = m * n, body = (count - p) & ~1;
-        pacer.wait(t, 8u * static_cast<uint32_t>(count), a.pace);
+        if (a.pace) pacer.wait(t, 8u * static_cast<uint32_t>(count));
         if (p) store_one<kPolicyStreaming>(row, b[1]);
         if ((count - p) & 1) store_one<kPolicyStreaming>(row + count - 1, b[p + count - 1]);
         if (body > 0) bulk_store(row + p, b + 2 * p, 8u * static_cast<uint32_t>(body));
@@ -842,8 +861,7 @@ __global__ void __launch_bounds__(kBlock) batch_work_kernel(const BatchWork *__r
 constexpr uint64_t kBulkUnitRows = 16;
 
 template <int VPT, int NB>
-__device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *buf, uint32_t &kb, uint32_t &warm,
-                                                  Pacer &pacer, uint32_t pace) {
+__device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *buf, uint32_t &kb, uint32_t &warm) {
   if (w.rows < kBulkUnitRows) {
     if (warm) {
       if (threadIdx.x == 0) bulk_wait_read<0>();
@@ -868,7 +886,8 @@ __device__ __forceinline__ void process_work_bulk(const BatchWork &w, uint64_t *
   a.ring_rows = 0;
   uint64_t st[VPT];
   load_tile<VPT, 1>(st, a, 0, w.count);
-  emit_rows_bulk<VPT, NB>(st, w.out + w.s_begin, w.streams, w.rows, w.count, 0, buf, kb, warm, pacer, pace);
+  Unpaced pacer;
+  emit_rows_bulk<VPT, NB>(st, w.out + w.s_begin, w.streams, w.rows, w.count, 0, buf, kb, warm, pacer);
 }
 
 template <int VPT, int NB>
@@ -877,11 +896,10 @@ __global__ void __launch_bounds__(kBlock) batch_work_bulk_kernel(const BatchWork
   extern __shared__ __align__(128) uint64_t bulk_buf[];
   static_assert(bulk_words<VPT, NB>() >= staged_words<VPT>(), "short units stage in the bulk buffers");
   uint32_t kb = 0, warm = 0;
-  Pacer pacer;
   if (counter == nullptr) {
     if (blockIdx.x < n) {
       const BatchWork w = work[blockIdx.x];
-      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm, pacer, 0);
+      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm);
     }
   } else {
     __shared__ uint32_t s_unit;
@@ -892,7 +910,7 @@ __global__ void __launch_bounds__(kBlock) batch_work_bulk_kernel(const BatchWork
       __syncthreads();
       if (u >= n) break;
       const BatchWork w = work[u];
-      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm, pacer, 0);
+      process_work_bulk<VPT, NB>(w, bulk_buf, kb, warm);
     }
   }
   if (threadIdx.x == 0) bulk_wait_all();
@@ -1063,12 +1081,12 @@ const void *select_rows_staged_t(uint32_t vpt) {
   }
 }
 
-template <bool BANDED, int OUT>
+template <bool BANDED, int OUT, bool RING = false>
 const void *select_rows_bulk_t(uint32_t vpt, uint32_t nb) {
-  if (vpt == 4 && nb == 8) return reinterpret_cast<const void *>(&rows_bulk_kernel<4, 8, BANDED, OUT>);
-  if (vpt == 8 && nb == 12) return reinterpret_cast<const void *>(&rows_bulk_kernel<8, 12, BANDED, OUT>);
-  if (vpt == 16 && nb == 6) return reinterpret_cast<const void *>(&rows_bulk_kernel<16, 6, BANDED, OUT>);
-  if (vpt == 24 && nb == 4) return reinterpret_cast<const void *>(&rows_bulk_kernel<24, 4, BANDED, OUT>);
+  if (vpt == 4 && nb == 8) return reinterpret_cast<const void *>(&rows_bulk_kernel<4, 8, BANDED, OUT, RING>);
+  if (vpt == 8 && nb == 12) return reinterpret_cast<const void *>(&rows_bulk_kernel<8, 12, BANDED, OUT, RING>);
+  if (vpt == 16 && nb == 6) return reinterpret_cast<const void *>(&rows_bulk_kernel<16, 6, BANDED, OUT, RING>);
+  if (vpt == 24 && nb == 4 && !RING) return reinterpret_cast<const void *>(&rows_bulk_kernel<24, 4, BANDED, OUT>);
   return nullptr;
 }
 
@@ -1084,6 +1102,11 @@ const void *select_rows_multi_t(uint32_t vpt) {
   }
 }
 
+const void *rows_bulk_ring_kernel_fn(uint32_t vpt, uint32_t nb, uint32_t out) {
+  return out == 1   ? select_rows_bulk_t<false, 1, true>(vpt, nb)
+         : out == 0 ? select_rows_bulk_t<false, 0, true>(vpt, nb)
+                    : nullptr;
+}
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out) {
   if (out == 1) return banded ? select_rows_bulk_t<true, 1>(vpt, nb) : select_rows_bulk_t<false, 1>(vpt, nb);
   if (out != 0) return nullptr;

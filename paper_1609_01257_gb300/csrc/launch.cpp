@@ -315,7 +315,8 @@ cudaError_t launch_rows(const RowsLaunch &a, const LaunchShape &sh, int store_po
   const int policy = store_policy == kStoreBulk ? kStoreStreaming : store_policy;
   const void *fn = bulk && sh.bulk.multi
                        ? (a.band_rows && a.pitch == a.s_end - a.s_begin ? rows_multi_kernel_fn(vpt, a.out_mode) : nullptr)
-                   : bulk   ? rows_bulk_kernel_fn(vpt, sh.bulk.nb, a.band_rows != 0, a.out_mode)
+                   : bulk   ? (a.ring_rows ? rows_bulk_ring_kernel_fn(vpt, sh.bulk.nb, a.out_mode)
+                                           : rows_bulk_kernel_fn(vpt, sh.bulk.nb, a.band_rows != 0, a.out_mode))
                    : staged ? rows_staged_kernel_fn(vpt, a.band_rows != 0, a.out_mode)
                             : rows_kernel_fn(vpt, width, policy, sh.block, a.band_rows != 0, a.out_mode);
   uint64_t grid = sh.grid;
