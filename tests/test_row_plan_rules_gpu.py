@@ -1,0 +1,36 @@
+"""Rules of the library's own plans for device rows, on both sides of each line:
+kernel and values per thread of the launch, and all values against the oracle,
+from the hash and then from states in memory."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1609_01257_gb300 as rng
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(n, T, off, kernel, vpt, mode=0):
+    buf = torch.full((T * n + off,), -1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()  # generate_to launches on the library's stream
+    g = rng.Generator(n, 71, output_mode=mode)
+    want = oracle.generate(n, 71, 2 * T, output_mode=mode)
+    for k in range(2):
+        g.generate_to(T, buf.data_ptr() + 8 * off)
+        g.sync()
+        got = buf.cpu().numpy().view(np.uint64)[off:].reshape(T, n)
+        assert np.array_equal(got, want[k * T:(k + 1) * T]), k
+    info = g.last_launch()
+    g.close()
+    assert (info["kernel"], info["values_per_thread"]) == (kernel, vpt)
+
+
+@pytest.mark.parametrize("n,T,off,kernel,vpt", [
+    (1 << 21, 16, 1, "bulk", 8),         # off the lines from 2^21 streams: bulk copies from 16 rows
+    (1 << 21, 31, 1, "bulk", 8),
+    (1 << 21, 15, 1, "staged", 1),
+    ((1 << 21) - 1, 31, 0, "staged", 2),
+])
+def test_few_rows_off_the_lines(n, T, off, kernel, vpt):
+    _check(n, T, off, kernel, vpt)
