@@ -119,9 +119,8 @@ uint32_t ceil16(uint64_t v) { return static_cast<uint32_t>((v + 15) / 16 * 16); 
 //    x 1024 188 / 154; below 128 rows register stores (direct_vpt) are faster;
 //  - 250001 x 255 81 / 82 (in bands 82), x 1024 293 / 281: from 1024 rows;
 //  - 400001 x 64 51 / 41, 1000003 x 128 167 / 150, 3000017 x 128 453 / 428, 2^22
-//    + 1 x 64 317 / 306; below 32 rows even or worse up to 2^21 streams, where
-//    the register stores of counts off the lines are (2^21 x 31 off a line 125
-//    staged / 89);
+//    + 1 x 64 317 / 306; below 32 rows even or worse up to 2^21 streams (2^21 x
+//    31 off a line 125 staged / 89);
 //  - on the lines, 2^20 x 255 307 / 292, 2^22 x 128 602 / 584, 65536 x 4096 293 /
 //    294 (and 340 where 128 unpaced SMs are past the ceiling); 2^22 x 64 308 /
 //    324, 2^24 x 32 656 / 690 (each tile's loads are exposed);
@@ -137,7 +136,7 @@ BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, u
   const uint64_t bytes = 8 * streams * out_rows;
   uint64_t units;
   if (streams <= 4096) {
-    if (!may_band || rows < (lined ? 16 * uint64_t(sms) : 64)) return p;
+    if (!may_band || rows < (lined ? 16 * uint64_t(sms) : streams % 16 == 0 && streams > 1024 ? 128 : 64)) return p;
     if (lined && streams > 1024 && bytes < 256 * M) return p;
     const uint64_t bands = std::min<uint64_t>(sms, rows / 16);
     p.multi = true;

@@ -34,3 +34,10 @@ def _check(n, T, off, kernel, vpt, mode=0):
 ])
 def test_few_rows_off_the_lines(n, T, off, kernel, vpt):
     _check(n, T, off, kernel, vpt)
+
+
+@pytest.mark.parametrize("n,T,kernel,vpt", [(4096, 64, "register", 1), (4096, 127, "register", 1),
+                                            (4096, 128, "bulk", 16), (1040, 127, "register", 1),
+                                            (1024, 64, "bulk", 4)])
+def test_few_streams_off_a_line(n, T, kernel, vpt):
+    _check(n, T, 1, kernel, vpt)
