@@ -28,10 +28,11 @@ const void *rows_kernel_fn(uint32_t vpt, int width, int policy, uint32_t block, 
 // 4, 6 or 8 values per thread, 256-thread blocks.
 const void *rows_staged_kernel_fn(uint32_t vpt, bool banded, uint32_t out);
 // Row kernel whose rows are written by TMA bulk copies from `nb` shared
-// buffers (4 values per thread with 8 buffers, 8 with 12, 16 with 6, 24 with
-// 4; 256-thread blocks), and its dynamic shared memory in bytes.
+// buffers (4 values per thread with 8 buffers, 8 with 12, 10 with 9, 16 with
+// 6, 24 with 4; 10 and 24 in the library's own plans only, 10 not banded;
+// 256-thread blocks), and its dynamic shared memory in bytes.
 const void *rows_bulk_kernel_fn(uint32_t vpt, uint32_t nb, bool banded, uint32_t out);
-const void *rows_bulk_ring_kernel_fn(uint32_t vpt, uint32_t nb, uint32_t out);  // rows wrap; vpt 4, 8 or 16
+const void *rows_bulk_ring_kernel_fn(uint32_t vpt, uint32_t nb, uint32_t out);  // rows wrap; vpt 4, 8, 10 or 16
 size_t rows_bulk_smem_bytes(uint32_t vpt, uint32_t nb);
 // Rings of more rows than this do not hold the bulk-copy row kernel up.
 constexpr int kBulkRingRows = 32;

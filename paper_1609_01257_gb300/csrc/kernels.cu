@@ -478,11 +478,11 @@ __device__ __forceinline__ void rows_bulk_units(const RowsLaunch &a, uint64_t *b
   if (threadIdx.x == 0) bulk_wait_all();
 }
 
-// Plans pace launches of 16 and 24 values per thread only (bulk_plan).
+// Plans pace launches of 10, 16 and 24 values per thread only (bulk_plan).
 template <int VPT, int NB, bool BANDED, int OUT = 0, bool RING = false>
 __global__ void __launch_bounds__(kBlock) rows_bulk_kernel(const RowsLaunch a) {
   extern __shared__ __align__(128) uint64_t bulk_buf[];
-  if constexpr (VPT >= 16) {
+  if constexpr (VPT >= 10) {
     if (a.pace) {
       rows_bulk_units<VPT, NB, BANDED, OUT, RING>(a, bulk_buf, Pacer{a.pace});
       return;
@@ -1085,6 +1085,7 @@ template <bool BANDED, int OUT, bool RING = false>
 const void *select_rows_bulk_t(uint32_t vpt, uint32_t nb) {
   if (vpt == 4 && nb == 8) return reinterpret_cast<const void *>(&rows_bulk_kernel<4, 8, BANDED, OUT, RING>);
   if (vpt == 8 && nb == 12) return reinterpret_cast<const void *>(&rows_bulk_kernel<8, 12, BANDED, OUT, RING>);
+  if (vpt == 10 && nb == 9 && !BANDED) return reinterpret_cast<const void *>(&rows_bulk_kernel<10, 9, false, OUT, RING>);
   if (vpt == 16 && nb == 6) return reinterpret_cast<const void *>(&rows_bulk_kernel<16, 6, BANDED, OUT, RING>);
   if (vpt == 24 && nb == 4 && !RING) return reinterpret_cast<const void *>(&rows_bulk_kernel<24, 4, BANDED, OUT>);
   return nullptr;

@@ -79,6 +79,7 @@ uint32_t bulk_buffers(uint32_t vpt) {
   switch (vpt) {
     case 4: return 8;
     case 8: return 12;
+    case 10: return 9;
     case 16: return 6;
     case 24: return 4;
     default: return 0;
@@ -109,12 +110,13 @@ uint32_t ceil16(uint64_t v) { return static_cast<uint32_t>((v + 15) / 16 * 16); 
 // tiles and bands come to whole rounds of the SMs, because a paced block does
 // not use what another leaves (1000003 streams x 512 rows, 16 values per
 // thread: 304 tiles of 3296 in two rounds 7555 GB/s, 245 of 4096 6106).  A
-// block's step per row takes about 0.3 us with 8 values per thread and 0.44
-// with 16, so tiles are as wide as the threads' values allow.
+// block's step per row takes about 0.3 us with 8 values per thread and 0.38
+// to 0.44 with 16, so tiles are as wide as the threads' values allow.
 // Where the lines lie (GB300, us before / with this plan):
 //  - up to 4096 streams, the whole row in a block: 300 x 100 44 / 14, 1001 x
 //    4096 60 / 18, 4096 x 65536 333 / 294; rows on the lines keep register
-//    stores below 256 MB (4096 x 4096 32 / 33) and 16 rows per band;
+//    stores below 256 MB (4096 x 4096 32 / 33) and 16 rows per band, and 4096 x
+//    64 off a line (9.9 / 19.8);
 //  - 5500 x 1024 74 / 24, 20001 x 16384 549 / 359, 65537 x 255 58 / 35, 131073
 //    x 1024 188 / 154; below 128 rows register stores (direct_vpt) are faster;
 //  - 250001 x 255 81 / 82 (in bands 82), x 1024 293 / 281: from 1024 rows;
@@ -178,6 +180,13 @@ BulkPlan bulk_plan(uint64_t streams, uint64_t rows, bool lined, bool may_band, u
       if (may_band) bands = std::max<uint64_t>(1, std::min<uint64_t>(sms / tiles, rows / 16));
       p.tile_w = ceil16((streams + sms / bands - 1) / (sms / bands));
       if (bands > 1) p.band_rows = (rows + bands - 1) / bands;
+    }
+    // Every value of a thread takes its time in a row, used or not: equal shares
+    // that come to at most 10 values run with 10 (622593 x 100 76 us, with 16
+    // values 97, staged 85; 330001 x 300 113 / 138).
+    if (bands == 1 && p.tile_w <= kGenBlock * 10) {
+      p.vpt = 10;
+      p.nb = bulk_buffers(p.vpt);
     }
     units = (streams + p.tile_w - 1) / p.tile_w * (bands > 1 ? (rows + p.band_rows - 1) / p.band_rows : 1);
   }

@@ -41,3 +41,33 @@ def test_few_rows_off_the_lines(n, T, off, kernel, vpt):
                                             (1024, 64, "bulk", 4)])
 def test_few_streams_off_a_line(n, T, kernel, vpt):
     _check(n, T, 1, kernel, vpt)
+
+
+@pytest.mark.parametrize("n,T,off,vpt", [
+    (311_297, 33, 0, 10),    # one tile a block
+    (389_120, 33, 1, 10),    # 2560 streams a tile: every value of a thread used
+    (389_121, 33, 0, 16),
+    (622_593, 40, 0, 10),    # two tiles a block
+    (778_240, 33, 1, 10),
+    (778_241, 33, 0, 16),
+    (1 << 20, 129, 0, 16),   # on the lines
+    (720_896, 129, 0, 10),
+])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_shares_of_at_most_ten_values(n, T, off, vpt, mode):
+    _check(n, T, off, "bulk", vpt, mode)
+
+
+@pytest.mark.parametrize("R", [1, 7, 8, 9, 32, 33])
+def test_rings_with_ten_values(R):
+    n, T = 330_001, 70
+    g = rng.Generator(n, 73)
+    ring = torch.zeros((R, n), dtype=torch.int64, device="cuda").view(torch.uint64)
+    g.generate_ring(T, ring)
+    got = ring.cpu().numpy()
+    info = g.last_launch()
+    g.close()
+    want = oracle.generate(n, 73, T)
+    assert (info["kernel"], info["values_per_thread"]) == ("bulk", 10)
+    for i in range(T - R, T):
+        assert np.array_equal(got[i % R], want[i]), i
