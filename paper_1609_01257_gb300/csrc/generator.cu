@@ -1046,10 +1046,8 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
     sh.vpt = vpt;
     sh.block = rngi::kGenBlock;
     uint64_t br = rngi::choose_band_rows(g->n, iterations, sh, g->device, true, a.out_mode);
-    if (!br && !capturing) {
-      br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
-      if (br && band_memory(g, static_cast<uint32_t>((iterations + br - 1) / br), !a.from_hash) != cudaSuccess) br = 0;
-    }
+    if (!br && !capturing) br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
+    if (br && band_memory(g, static_cast<uint32_t>((iterations + br - 1) / br), !a.from_hash) != cudaSuccess) br = 0;
     if (br) {
       rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
       if (rc) return rc;
