@@ -314,7 +314,13 @@ int rng_get_state(rng_gen *g, uint64_t *host_states, rng_err **err);
 int rng_set_state(rng_gen *g, const uint64_t *host_states, uint64_t position, rng_err **err);
 /* Waits for all work the generator has queued. */
 int rng_sync(rng_gen *g, rng_err **err);
-/* The compute stream (cudaStream_t) the generator launches on. */
+/* The compute stream (cudaStream_t) the generator launches on.  Device output,
+ * checksums and rng_skip can be captured on it into a graph (with
+ * rng_opts.profiling 0): a replay goes on from the states that the work before
+ * it left, or from the ids where rng_init is part of the capture; the position
+ * that rng_position gives counts the calls, not the replays.  A capture
+ * allocates nothing: a launch that would be split by rows is split only if the
+ * same call has run before on this generator. */
 void *rng_compute_stream(rng_gen *g);
 /* Order the generator's work with a stream of the caller's (a cudaStream_t of
  * the same device), by an event: what the generator launches next starts

@@ -65,7 +65,9 @@ struct rng_gen {
   uint64_t jump_rows = 0;            // band_rows the table on the device is for
   uint32_t jump_count = 0;           // bands in that table
   uint32_t jump_cap = 0;             // bands it has room for
-  uint64_t *d_jump_small = nullptr;  // the table before it grew
+  bool jump_in_graph = false;        // a captured launch reads that table: it stays as it is
+  std::vector<uint64_t *> old_jump;  // tables that launches or graphs may still read
+  bool captured = false;             // a launch was recorded into a graph (see capturing())
   cudaStream_t compute = nullptr, copy = nullptr;
   bool own_compute = false;
   uint64_t *d_buf[2] = {nullptr, nullptr};
@@ -145,52 +147,65 @@ int profile_restart(rng_gen *g, rng_err **err) {
   return rngi::cuda_fail(err, cudaEventRecord(g->origin, g->compute), "cudaEventRecord");
 }
 
-// Device memory of a launch in `bands` bands: the jump tables and, with
-// `second_state`, the second state array.  Sized for what is asked (a table
-// for every SM's band is 320 KB, which cudaMalloc gives in microseconds where
-// 2 MB take about 100), so a generator's first banded launch does not wait
-// for it.
-cudaError_t band_memory(rng_gen *g, uint32_t bands, bool second_state) {
-  if (second_state && !g->d_state2) {
-    const cudaError_t e = cudaMalloc(&g->d_state2, g->n * 8);
-    if (e != cudaSuccess) {
-      g->d_state2 = nullptr;
-      cudaGetLastError();
-      return e;
-    }
-  }
-  if (g->jump_cap < bands) {
-    const uint32_t cap = bands <= 160 ? 160 : rngi::kMaxBands;
-    uint64_t *p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, size_t(cap) * rngi::kJumpTableWords * 8);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e;
-    }
-    g->d_jump_small = g->d_jump;  // launches in flight may read it: freed with the generator
-    g->d_jump = p;
-    g->jump_cap = cap;
-    g->jump_rows = 0;
-  }
-  return cudaSuccess;
+// Whether the compute stream is being captured into a graph.  Replays use the
+// state array by address, so from the first capture on final states come back
+// to it instead of the two arrays changing places.  Any call that queues work
+// on the states asks this first.
+bool capturing(rng_gen *g) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool on = cudaStreamIsCapturing(g->compute, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (on) g->captured = true;
+  return on;
 }
 
-// Prepares a banded launch of `a` with `br` rows per band: the jump tables on
-// the device and, where blocks read starting states that others replace
-// (second_state), the second state array (final states go there; the
-// generator switches to it after the launch).
-int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state, bool *swap, rng_err **err) {
+// Whether a launch of `rows` rows in bands of `br` can have its memory: the jump
+// tables and, with `second_state`, the second state array.  Without them the
+// launch runs unbanded, slower, but that is not an error.  Sized for what is
+// asked (a table for every SM's band is 320 KB, which cudaMalloc gives in
+// microseconds where 2 MB take about 100), so a generator's first banded launch
+// does not wait for it.  Under capture nothing is allocated and no table is
+// computed (the graph would not have run when the next launch looks for it):
+// bands only with what an eager launch of the same length has left.
+bool can_band(rng_gen *g, uint64_t rows, uint64_t br, bool second_state, bool under_capture) {
+  const uint32_t bands = static_cast<uint32_t>(std::min<uint64_t>((rows + br - 1) / br, rngi::kMaxBands));
+  const bool there = g->jump_rows == br && g->jump_count >= bands;
+  if (under_capture) return there && (!second_state || g->d_state2);
+  if (second_state && !g->d_state2 && cudaMalloc(&g->d_state2, g->n * 8) != cudaSuccess) {
+    g->d_state2 = nullptr;
+    cudaGetLastError();
+    return false;
+  }
+  if (there || (g->jump_cap >= bands && !g->jump_in_graph)) return true;
+  const uint32_t cap = bands <= 160 ? 160 : rngi::kMaxBands;
+  uint64_t *p = nullptr;
+  if (cudaMalloc(&p, size_t(cap) * rngi::kJumpTableWords * 8) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (g->d_jump) g->old_jump.push_back(g->d_jump);
+  g->d_jump = p;
+  g->jump_cap = cap;
+  g->jump_rows = g->jump_count = 0;
+  g->jump_in_graph = false;
+  return true;
+}
+
+// Prepares a banded launch of `a` with `br` rows per band, for which can_band
+// gave the memory: the jump tables on the device and, where blocks read
+// starting states that others replace (second_state), the second state array
+// (final states go there, and adopt_states makes them the generator's).
+int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state, bool under_capture, bool *swap,
+                rng_err **err) {
   const uint64_t bands = (a.rows + br - 1) / br;
   if (bands > rngi::kMaxBands) return rngi::fail(err, RNG_EINVAL, "banded launch: %llu bands", (unsigned long long)bands);
   const uint32_t count = static_cast<uint32_t>(bands);
-  int rc = rngi::cuda_fail(err, band_memory(g, count, second_state), "cudaMalloc(second state array, jump tables)");
-  if (rc) return rc;
   if (g->jump_rows != br || g->jump_count < count) {
-    rc = rngi::cuda_fail(err, rngi::launch_jump_tables(g->d_jump, br, count, g->compute), "jump table launch");
+    const int rc = rngi::cuda_fail(err, rngi::launch_jump_tables(g->d_jump, br, count, g->compute), "jump table launch");
     if (rc) return rc;
     g->jump_rows = br;
     g->jump_count = count;
   }
+  if (under_capture) g->jump_in_graph = true;
   a.band_rows = br;
   a.jump = g->d_jump;
   if (a.write_state && second_state) {
@@ -200,11 +215,18 @@ int setup_bands(rng_gen *g, rngi::RowsLaunch &a, uint64_t br, bool second_state,
   return RNG_OK;
 }
 
+// After a launch that left the final states in the second array.
+cudaError_t adopt_states(rng_gen *g) {
+  if (g->captured)
+    return cudaMemcpyAsync(g->d_state, g->d_state2, g->n * 8, cudaMemcpyDeviceToDevice, g->compute);
+  std::swap(g->d_state, g->d_state2);
+  return cudaSuccess;
+}
+
 // Launches the row kernel for `a`.  When the launch covers every stream but
 // has too few tiles to fill the GPU, its rows are split into bands run by
 // separate blocks: each band's blocks jump their states ahead over GF(2),
-// and the final states are written to the second state array, which then
-// becomes the current one.
+// and the final states are written to the second state array.
 // device_out: a.out is device memory (the bulk-copy kernel may write it);
 // host destinations keep the register-store kernels.
 int gen_launch_rows(rng_gen *g, rngi::RowsLaunch &a, const rngi::LaunchShape &shape, bool device_out,
@@ -218,32 +240,24 @@ int gen_launch_rows(rng_gen *g, rngi::RowsLaunch &a, const rngi::LaunchShape &sh
     base.bulk_auto = false;
     base.bulk_forced = false;
   }
-  // Never under capture: the second state array would be allocated, and a
-  // replay would not find the arrays swapped.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool may_band = !a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n &&
-                        cudaStreamIsCapturing(g->compute, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  const bool under_capture = capturing(g);
+  const bool may_band = !a.ring_rows && a.out && a.s_begin == 0 && a.s_end == g->n;
   rngi::LaunchShape sh = rngi::resolve_shape(base, a, may_band);
   bool swap = false;
   if (may_band) {
-    uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
-    if (br && band_memory(g, static_cast<uint32_t>(std::min<uint64_t>((a.rows + br - 1) / br, rngi::kMaxBands)),
-                          !a.from_hash) != cudaSuccess) {
-      // No memory for bands: slower without them, but not an error.
+    const uint64_t br = rngi::choose_band_rows(g->n, a.rows, sh, g->device, false, a.out_mode);
+    if (br && !can_band(g, a.rows, br, !a.from_hash, under_capture)) {
       sh = rngi::resolve_shape(base, a, false);
-      br = 0;
-    }
-    if (br) {
-      int rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
+    } else if (br) {
+      int rc = setup_bands(g, a, br, !a.from_hash, under_capture, &swap, err);
       if (rc) return rc;
     }
   }
   long op = op_begin(g, "RNG_KERNEL", kQueueMain, g->compute);
   cudaError_t st = rngi::launch_rows(a, sh, static_cast<int>(g->opts.store_policy), g->compute, &g->last_launch);
   op_end(g, op, g->compute);
-  int rc = rngi::cuda_fail(err, st, "rows kernel launch");
-  if (!rc && swap) std::swap(g->d_state, g->d_state2);
-  return rc;
+  if (st == cudaSuccess && swap) st = adopt_states(g);
+  return rngi::cuda_fail(err, st, "rows kernel launch");
 }
 
 // Device buffers and events of the double buffer; with `slots` > 0, at least
@@ -810,7 +824,7 @@ void rng_destroy(rng_gen *g) {
   cudaFree(g->d_state);
   cudaFree(g->d_state2);
   cudaFree(g->d_jump);
-  cudaFree(g->d_jump_small);
+  for (uint64_t *p : g->old_jump) cudaFree(p);
   for (int b = 0; b < 2; ++b) {
     cudaFree(g->d_buf[b]);
     if (g->produced[b]) cudaEventDestroy(g->produced[b]);
@@ -834,6 +848,7 @@ int rng_init(rng_gen *g, rng_err **err) {
   g->pos = 0;
   g->materialized = false;
   if (!g->opts.fuse_init) {
+    capturing(g);
     long op = op_begin(g, "INIT_KERNEL", kQueueMain, g->compute);
     cudaError_t st = rngi::launch_init(g->d_state, g->n, g->g0, g->key, g->compute);
     op_end(g, op, g->compute);
@@ -1019,21 +1034,16 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   a.out_mode = g->opts.output_mode;
   bool swap = false;
   long op = -1;
-  // Launches that fill the GPU are split by rows except where a capture would
-  // record one of two state arrays.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool capturing = cudaStreamIsCapturing(g->compute, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  const bool under_capture = capturing(g);
   rngi::SlicedPlan plan;
   if (!g->opts.values_per_thread && a.out_mode == 0) {
-    plan = rngi::choose_sliced(g->n, iterations, g->device, !capturing);
-    if (plan.quantum_rows &&
-        band_memory(g, static_cast<uint32_t>((iterations + plan.quantum_rows - 1) / plan.quantum_rows), !a.from_hash) !=
-            cudaSuccess)
+    plan = rngi::choose_sliced(g->n, iterations, g->device, true);
+    if (plan.quantum_rows && !can_band(g, iterations, plan.quantum_rows, !a.from_hash, under_capture))
       plan = rngi::choose_sliced(g->n, iterations, g->device, false);
   }
   if (plan.blocks) {
     if (plan.quantum_rows) {
-      rc = setup_bands(g, a, plan.quantum_rows, !a.from_hash, &swap, err);
+      rc = setup_bands(g, a, plan.quantum_rows, !a.from_hash, under_capture, &swap, err);
       if (rc) return rc;
     }
     op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
@@ -1041,24 +1051,24 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
   } else {
     const uint32_t v = g->opts.values_per_thread;
     const uint32_t vpt = rngi::checksum_vpt(g->n, iterations, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0);
-    // Few tiles, many rows: bands, as for the row kernel.
+    // Few tiles, many rows: bands, as for the row kernel.  Launches that fill
+    // the GPU are split by rows where that fills the last wave.
     rngi::LaunchShape sh{};
     sh.vpt = vpt;
     sh.block = rngi::kGenBlock;
     uint64_t br = rngi::choose_band_rows(g->n, iterations, sh, g->device, true, a.out_mode);
-    if (!br && !capturing) br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
-    if (br && band_memory(g, static_cast<uint32_t>((iterations + br - 1) / br), !a.from_hash) != cudaSuccess) br = 0;
-    if (br) {
-      rc = setup_bands(g, a, br, !a.from_hash, &swap, err);
+    if (!br) br = rngi::checksum_split_rows(g->n, iterations, vpt, g->device, a.out_mode);
+    if (br && can_band(g, iterations, br, !a.from_hash, under_capture)) {
+      rc = setup_bands(g, a, br, !a.from_hash, under_capture, &swap, err);
       if (rc) return rc;
     }
     op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
     st = rngi::launch_checksum(a, vpt, row_xor_dev, row_sum_dev, g->compute);
   }
   op_end(g, op, g->compute);
+  if (st == cudaSuccess && swap) st = adopt_states(g);
   rc = rngi::cuda_fail(err, st, "checksum kernel launch");
   if (rc) return rc;
-  if (swap) std::swap(g->d_state, g->d_state2);
   g->materialized = true;
   g->pos += iterations;
   return RNG_OK;
@@ -1071,6 +1081,7 @@ int rng_skip(rng_gen *g, uint64_t iterations, rng_err **err) {
   if (iterations == 0) return RNG_OK;
   uint64_t cols[64];
   rngi::jump_matrix(iterations, cols);  // on the host, before the timed op
+  capturing(g);
   long op = op_begin(g, "SKIP_KERNEL", kQueueMain, g->compute);
   cudaError_t st = rngi::launch_jump(g->d_state, g->n, g->g0, g->key, !g->materialized, cols, g->compute);
   op_end(g, op, g->compute);
