@@ -342,7 +342,13 @@ int rng_launch_config(const rng_gen *g, uint32_t *values_per_thread,
  * shared memory and written by TMA bulk copies, row_buffers buffers in turn).
  * band_rows: rows per band of a banded launch, else 0.  Set info->struct_size
  * = sizeof(rng_launch_info) first.  RNG_ESTATE before the first launch. */
-enum { RNG_KERNEL_REGISTER = 0, RNG_KERNEL_STAGED = 1, RNG_KERNEL_BULK = 2 };
+enum {
+    RNG_KERNEL_REGISTER = 0,
+    RNG_KERNEL_STAGED = 1,
+    RNG_KERNEL_BULK = 2,
+    RNG_KERNEL_CHECKSUM = 3, /* rng_last_checksum */
+    RNG_KERNEL_SLICED = 4
+};
 typedef struct rng_launch_info {
     uint32_t struct_size;
     uint32_t kernel;
@@ -353,6 +359,10 @@ typedef struct rng_launch_info {
     uint64_t band_rows;
 } rng_launch_info;
 int rng_last_launch(const rng_gen *g, rng_launch_info *info, rng_err **err);
+/* The same of the last rng_generate_checksum: RNG_KERNEL_CHECKSUM or, bit
+ * planes of 32 streams a word, RNG_KERNEL_SLICED.  band_rows: the rows that
+ * tiles are split by, 0 = whole tiles; row_buffers 0. */
+int rng_last_checksum(const rng_gen *g, rng_launch_info *info, rng_err **err);
 
 /* Releases the device state, buffers, streams and events.  NULL-safe. */
 void rng_destroy(rng_gen *g);

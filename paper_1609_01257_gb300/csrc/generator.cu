@@ -58,6 +58,7 @@ struct rng_gen {
   rngi::LaunchShape shape{};
   rngi::LaunchShape chunk_shape{};  // shape of the last streamed chunk width
   rngi::LaunchInfo last_launch{};   // what the last row-kernel launch ran
+  rngi::LaunchInfo last_checksum{};  // what the last generate-and-checksum launch ran
   uint64_t chunk_span = 0;
   uint64_t *d_state = nullptr;
   uint64_t *d_state2 = nullptr;      // second state array for banded launches
@@ -1047,7 +1048,7 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
       if (rc) return rc;
     }
     op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
-    st = rngi::launch_checksum_sliced(a, plan, row_xor_dev, row_sum_dev, g->compute);
+    st = rngi::launch_checksum_sliced(a, plan, row_xor_dev, row_sum_dev, g->compute, &g->last_checksum);
   } else {
     const uint32_t v = g->opts.values_per_thread;
     const uint32_t vpt = rngi::checksum_vpt(g->n, iterations, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0);
@@ -1063,7 +1064,7 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
       if (rc) return rc;
     }
     op = op_begin(g, "CHECKSUM_KERNEL", kQueueMain, g->compute);
-    st = rngi::launch_checksum(a, vpt, row_xor_dev, row_sum_dev, g->compute);
+    st = rngi::launch_checksum(a, vpt, row_xor_dev, row_sum_dev, g->compute, &g->last_checksum);
   }
   op_end(g, op, g->compute);
   if (st == cudaSuccess && swap) st = adopt_states(g);
@@ -1176,13 +1177,13 @@ int rng_launch_config(const rng_gen *g, uint32_t *vpt, uint32_t *block, uint32_t
   return RNG_OK;
 }
 
-int rng_last_launch(const rng_gen *g, rng_launch_info *info, rng_err **err) {
-  if (!g || !info) return rngi::fail(err, RNG_EINVAL, "rng_last_launch: NULL generator or info");
+static int launch_info(const rng_gen *g, const rngi::LaunchInfo rng_gen::*of, const char *fn, rng_launch_info *info,
+                       rng_err **err) {
+  if (!g || !info) return rngi::fail(err, RNG_EINVAL, "%s: NULL generator or info", fn);
   if (info->struct_size != sizeof(rng_launch_info))
-    return rngi::fail(err, RNG_EINVAL, "rng_last_launch: info.struct_size %u != %zu", info->struct_size,
-                      sizeof(rng_launch_info));
-  const rngi::LaunchInfo &l = g->last_launch;
-  if (l.block == 0) return rngi::fail(err, RNG_ESTATE, "rng_last_launch: no row-kernel launch yet");
+    return rngi::fail(err, RNG_EINVAL, "%s: info.struct_size %u != %zu", fn, info->struct_size, sizeof(rng_launch_info));
+  const rngi::LaunchInfo &l = g->*of;
+  if (l.block == 0) return rngi::fail(err, RNG_ESTATE, "%s: no such launch yet", fn);
   info->kernel = l.kernel;
   info->values_per_thread = l.vpt;
   info->block_threads = l.block;
@@ -1190,6 +1191,14 @@ int rng_last_launch(const rng_gen *g, rng_launch_info *info, rng_err **err) {
   info->row_buffers = l.row_buffers;
   info->band_rows = l.band_rows;
   return RNG_OK;
+}
+
+int rng_last_launch(const rng_gen *g, rng_launch_info *info, rng_err **err) {
+  return launch_info(g, &rng_gen::last_launch, "rng_last_launch", info, err);
+}
+
+int rng_last_checksum(const rng_gen *g, rng_launch_info *info, rng_err **err) {
+  return launch_info(g, &rng_gen::last_checksum, "rng_last_checksum", info, err);
 }
 
 rng_prof *rng_profiler(rng_gen *g, rng_err **err) {

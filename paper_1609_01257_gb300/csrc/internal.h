@@ -112,7 +112,7 @@ struct LaunchShape {
   BulkPlan bulk;            // set by resolve_shape: what this launch runs
 };
 
-// What one row-kernel launch ran (rng_launch_info without struct_size).
+// What one launch ran (rng_launch_info without struct_size).
 struct LaunchInfo {
   uint32_t kernel = 0;
   uint32_t vpt = 0, block = 0, grid = 0, row_buffers = 0;
@@ -164,7 +164,7 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt);
 // Generate-and-checksum launch with `vpt` values per thread; a.band_rows != 0
 // selects the banded variant (a.jump, a.state_out as for the row kernel).
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,
-                            cudaStream_t st);
+                            cudaStream_t st, LaunchInfo *info);
 // How a generate-and-checksum launch runs bit-sliced: `blocks` blocks over
 // equal runs of (tile, quantum of `quantum_rows` rows) pairs; quantum_rows ==
 // 0: whole tiles; blocks == 0: the launch keeps checksum_kernel.
@@ -177,7 +177,7 @@ struct SlicedPlan {
 SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_split);
 // a.band_rows = the plan's quantum_rows.
 cudaError_t launch_checksum_sliced(const RowsLaunch &a, const SlicedPlan &plan, uint64_t *row_xor, uint64_t *row_sum,
-                                   cudaStream_t st);
+                                   cudaStream_t st, LaunchInfo *info);
 int device_sm_count(int device);
 
 // Work-list kernel tables (batched and served forms).  One entry is a chunk

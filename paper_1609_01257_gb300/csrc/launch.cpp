@@ -475,7 +475,7 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
 }
 
 cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor, uint64_t *row_sum,
-                            cudaStream_t st) {
+                            cudaStream_t st, LaunchInfo *info) {
   const uint64_t span = a.s_end - a.s_begin;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -492,7 +492,10 @@ cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor
   unsigned long long *rs = reinterpret_cast<unsigned long long *>(row_sum);
   void *params[] = {&args, &rx, &rs};
   cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(kGenBlock), params, 0, st);
-  if (e == cudaSuccess) count_launch();
+  if (e == cudaSuccess) {
+    count_launch();
+    *info = {RNG_KERNEL_CHECKSUM, vpt, kGenBlock, grid, 0, a.band_rows};
+  }
   return e;
 }
 
@@ -533,14 +536,17 @@ SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_s
 }
 
 cudaError_t launch_checksum_sliced(const RowsLaunch &a, const SlicedPlan &plan, uint64_t *row_xor, uint64_t *row_sum,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, LaunchInfo *info) {
   if (!plan.blocks || (a.band_rows && !a.jump)) return cudaErrorInvalidValue;
   RowsLaunch args = a;
   unsigned long long *rx = reinterpret_cast<unsigned long long *>(row_xor);
   unsigned long long *rs = reinterpret_cast<unsigned long long *>(row_sum);
   void *params[] = {&args, &rx, &rs};
   cudaError_t e = cudaLaunchKernel(checksum_sliced_kernel_fn(), dim3(plan.blocks), dim3(kSlicedBlock), params, 0, st);
-  if (e == cudaSuccess) count_launch();
+  if (e == cudaSuccess) {
+    count_launch();
+    *info = {RNG_KERNEL_SLICED, uint32_t(kSlicedTile / kSlicedBlock), kSlicedBlock, plan.blocks, 0, a.band_rows};
+  }
   return e;
 }
 

@@ -127,9 +127,17 @@ class Generator:
         """What the last row-kernel launch ran: kernel ("register", "staged"
         or "bulk"), values per thread, block, grid, bulk row buffers and band
         rows (0 = unbanded)."""
+        return self._launch_info(self._lib.rng_last_launch)
+
+    def last_checksum(self) -> dict:
+        """The same of the last ``generate_checksum``: kernel "checksum" or
+        "sliced", band rows the rows that tiles are split by (0 = whole)."""
+        return self._launch_info(self._lib.rng_last_checksum)
+
+    def _launch_info(self, fn) -> dict:
         info = C.RngLaunchInfo()
         info.struct_size = ctypes.sizeof(C.RngLaunchInfo)
-        C.check(self._lib.rng_last_launch, self._h, ctypes.byref(info))
+        C.check(fn, self._h, ctypes.byref(info))
         return {"kernel": C.KERNEL_NAMES.get(info.kernel, str(info.kernel)),
                 "values_per_thread": info.values_per_thread, "block": info.block_threads,
                 "grid": info.grid_blocks, "row_buffers": info.row_buffers, "band_rows": info.band_rows}
