@@ -1051,7 +1051,7 @@ int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev
     st = rngi::launch_checksum_sliced(a, plan, row_xor_dev, row_sum_dev, g->compute, &g->last_checksum);
   } else {
     const uint32_t v = g->opts.values_per_thread;
-    const uint32_t vpt = rngi::checksum_vpt(g->n, iterations, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0);
+    const uint32_t vpt = rngi::checksum_vpt(g->n, iterations, (v && (v & (v - 1)) == 0 && v <= 64) ? v : 0, g->device);
     // Few tiles, many rows: bands, as for the row kernel.  Launches that fill
     // the GPU are split by rows where that fills the last wave.
     rngi::LaunchShape sh{};

@@ -452,8 +452,9 @@ uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int 
   return band;
 }
 
-uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
+uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt, int device) {
   if (vpt) return vpt;
+  const uint64_t sms = static_cast<uint64_t>(device_sm_count(device));
   // Large launches run at the ALU rate with 8 to 32 values per thread; the
   // start of a unit (jump, reductions) weighs least at 16.  Small launches are
   // bound by one block's rows, one after another, so they take fewer values
@@ -462,9 +463,9 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt) {
   // 62 / 62 / 60; 65536 x 4096 176 / 167 / 173) unless there are many tiles
   // anyway.  A tile that would be mostly past the end of the streams is halved.
   const uint64_t values = span * rows;
-  uint32_t v = values >= (uint64_t(1) << 26)                              ? 16
-               : values >= (uint64_t(1) << 24) || span >= 256 * 8 * 152 ? 8
-                                                                          : 4;
+  uint32_t v = values >= (uint64_t(1) << 26)                                 ? 16
+               : values >= (uint64_t(1) << 24) || span >= kGenBlock * 8 * sms ? 8
+                                                                              : 4;
   while (v > 1) {
     const uint64_t tile = uint64_t(kGenBlock) * v, tiles = (span + tile - 1) / tile;
     if (span * 5 >= tiles * tile * 4) break;
