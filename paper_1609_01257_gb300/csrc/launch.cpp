@@ -1,15 +1,13 @@
 // Host-side launch code of the kernels: shape selection (values per thread,
 // store width, grid, bands) and the launches themselves, but for the
-// jump-ahead's (jump.cu).  The kernels are in
-// kernels.cu; this file holds no device code.
+// jump-ahead's (jump.cu).  The kernels are in kernels.cu and
+// checksum_sliced.cu; this file holds no device code.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "internal.h"
-#include "prng_math.cuh"
 
 namespace rngi {
 namespace {
@@ -91,7 +89,10 @@ namespace {
 // Blocks that write at the same time hold their copies to this rate (bytes a
 // second, all together): see Pacer.  With 152 blocks and 2^22 streams x 256
 // rows 7.5, 7.6, 7.7 and 7.8e12 gave 7422, 7518, 7621 and 7711 GB/s; a
-// copy-only kernel held 7.88e12 and fell back at 8.0e12.
+// copy-only kernel held 7.88e12 and fell back at 8.0e12.  For the whole GB300
+// (HBM3e, 7.9 TB/s nominal; fills 7.55 to 7.65 on those measured): on a
+// partition, or a part whose memory takes less, the pace does not hold the
+// copies back and they run as they did without it.
 constexpr double kWriteRate = 7.7e12;
 
 uint32_t pace_of(uint64_t blocks) {
@@ -433,6 +434,7 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
 }
 
 uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int device, uint32_t out) {
+  if (rows < 2 * 64) return 0;  // before the occupancy query, a microsecond of the host
   const uint64_t tile = uint64_t(kGenBlock) * vpt, tiles = (streams + tile - 1) / tile;
   const void *fn = checksum_kernel_fn(vpt, true, out);
   if (!fn) return 0;
@@ -503,7 +505,10 @@ cudaError_t launch_checksum(const RowsLaunch &a, uint32_t vpt, uint64_t *row_xor
 SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_split) {
   SlicedPlan p;
   const uint64_t tiles = (streams + kSlicedTile - 1) / kSlicedTile;
-  // A partly filled last tile costs as much as a full one.
+  // A partly filled last tile costs as much as a full one, and the other kernel
+  // has smaller tiles: one tile at two thirds 118 / 109 us for 2^27 values and
+  // 615 / 649 for 2^30, at 0.72 108 / 107 and 572 / 606, full 92 / 97 and 425 /
+  // 551; two and three tiles the same within 4 %.
   if (streams * 3 < tiles * kSlicedTile * 2) return p;
   // Each tile pays for its states' way into bit planes and back, and small
   // launches need more blocks than there are tiles: us bit-sliced / best
@@ -517,8 +522,8 @@ SlicedPlan choose_sliced(uint64_t streams, uint64_t rows, int device, bool may_s
   const double whole = static_cast<double>(tiles) / static_cast<double>(waves * slots);  // share of the slots in use
   p.blocks = static_cast<uint32_t>(std::min(tiles, uint64_t(0x7fffffff)));
   if (!may_split || whole > 0.97) return p;
-  // The fewest quanta per tile (each is one matrix to compute and upload)
-  // that leave the longest run within 3 % of the mean; at least 16 rows each.
+  // The fewest quanta per tile (each has its jump tables, one block's work) that
+  // leave the longest run within 3 % of the mean; at least 16 rows each.
   double best = whole;
   for (uint64_t nq = 2; nq <= std::min<uint64_t>(rows / 16, kMaxBands); ++nq) {
     const uint64_t q = (rows + nq - 1) / nq;
