@@ -54,10 +54,17 @@ WORKLOADS = {
                   name="plain method: 2^16 streams x 100 iterations, seed 0"),
 }
 
-# ALU-pipe lane operations per value of the generate-and-checksum kernels on
-# large launches in output modes 0 (bit-sliced) and 1, from their ncu captures:
-# ALU-pipe warp instructions x 32 / values over 2^22 streams x 512 and 64 rows.
-CHECKSUM_ALU_OPS_PER_VALUE = {0: 5.95, 1: 9.43}
+# ALU-pipe lane operations per value of the generate-and-checksum kernels, from
+# their ncu captures (ALU-pipe warp instructions x 32 / values): by output mode
+# the kernel, the fewest rows of 2^22 streams that the figure stands for, and
+# the figure.  Fewer streams or rows run more per value (the start of a tile).
+CHECKSUM_ALU_OPS = {0: ("sliced", 512, 5.95), 1: ("checksum", 64, 9.43)}
+
+
+def checksum_alu_ops(mode: int, kernel: str, streams: int, rows: int) -> float | None:
+    """The captured figure when the run is of its kernel and size, else None."""
+    k, least, ops = CHECKSUM_ALU_OPS[mode]
+    return ops if kernel == k and streams >= 1 << 22 and rows >= least else None
 NOMINAL_HBM_GBPS = 7900.0  # GB300 HBM3e, nominal
 METRIC = "GB/s of uint64 PRNG output (device and host-streamed) vs roofline; p50/p99 req latency"
 
@@ -847,6 +854,7 @@ def checksum_leg(args, wl, clocks=None):
     secs = e0.elapsed_time(e1) * 1e-3
     clk = clocks.stop(t_start, t_end) if own else clocks.window(t_start, t_end)
     c, t = g.profile_stat("CHECKSUM_KERNEL")
+    kernel = g.last_checksum()["kernel"]
     g.close()
     props = torch.cuda.get_device_properties(0)
     vps = n * T * args.steps / secs
@@ -856,15 +864,15 @@ def checksum_leg(args, wl, clocks=None):
     # duration / values).
     sm_mhz = (clk or {}).get("sm_mhz") or 2070.0  # nominal maximum when nvidia-smi gave no sample
     peak = props.multi_processor_count * 64 * sm_mhz * 1e6 / 1e12
-    ops = CHECKSUM_ALU_OPS_PER_VALUE[args.output_mode]
-    achieved = vps * ops / 1e12
+    ops = checksum_alu_ops(args.output_mode, kernel, n, T)
+    achieved = vps * ops / 1e12 if ops else None
     return {"config": {"workload": wl["name"] + " (generate-and-checksum mode)" + _mode_label(args),
                        "streams": n, "iterations": T, "seed": seed},
             "values_per_s": vps,
             "equiv_GBps": 8 * vps / 1e9, "kernel_avg_ms": 1e3 * t / max(c, 1), "steps": args.steps,
-            "sms": props.multi_processor_count,
+            "sms": props.multi_processor_count, "kernel": kernel,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s (ALU-pipe lane ops)",
-                         "frac": achieved / peak, "alu_ops_per_value": ops,
+                         "frac": achieved / peak if ops else None, "alu_ops_per_value": ops,
                          "peak_source": "SMs x 64 ALU-pipe lanes x median SM clock during the timed region"},
             "clocks": clk}
 
