@@ -434,7 +434,7 @@ uint64_t choose_band_rows(uint64_t streams, uint64_t rows, const LaunchShape &sh
 }
 
 uint64_t checksum_split_rows(uint64_t streams, uint64_t rows, uint32_t vpt, int device, uint32_t out) {
-  if (rows < 2 * 64) return 0;  // before the occupancy query, a microsecond of the host
+  if (rows < 2 * 64) return 0;  // before the occupancy query, 0.2 us of the host
   const uint64_t tile = uint64_t(kGenBlock) * vpt, tiles = (streams + tile - 1) / tile;
   const void *fn = checksum_kernel_fn(vpt, true, out);
   if (!fn) return 0;
@@ -463,11 +463,14 @@ uint32_t checksum_vpt(uint64_t span, uint64_t rows, uint32_t vpt, int device) {
   // per thread and more blocks (us on GB300 at 4 / 8 / 16: 8192 x 1024 25 / 30
   // / 40; 65536 x 256 32 / 31 / 40; 1000003 x 16 37 / 27 / 29; 262144 x 256
   // 62 / 62 / 60; 65536 x 4096 176 / 167 / 173) unless there are many tiles
-  // anyway.  A tile that would be mostly past the end of the streams is halved.
+  // anyway: many tiles of few rows wait for their atomics on the same few
+  // words, so from five tiles of 16 values an SM on the larger ones are taken (8
+  // / 16: 2^22 x 15 50 / 43, 6000001 x 8 42 / 35).  A tile that would be mostly past
+  // the end of the streams is halved.
   const uint64_t values = span * rows;
-  uint32_t v = values >= (uint64_t(1) << 26)                                 ? 16
-               : values >= (uint64_t(1) << 24) || span >= kGenBlock * 8 * sms ? 8
-                                                                              : 4;
+  uint32_t v = values >= (uint64_t(1) << 26) || span >= kGenBlock * 16 * 5 * sms ? 16
+               : values >= (uint64_t(1) << 24) || span >= kGenBlock * 8 * sms    ? 8
+                                                                                 : 4;
   while (v > 1) {
     const uint64_t tile = uint64_t(kGenBlock) * v, tiles = (span + tile - 1) / tile;
     if (span * 5 >= tiles * tile * 4) break;

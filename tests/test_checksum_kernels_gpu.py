@@ -79,6 +79,18 @@ def test_launches_beside_the_line_take_the_other_kernel(n, rows, kw):
     _same(got, n, 79, rows, output_mode=kw.get("output_mode", 0))
 
 
+@pytest.mark.parametrize("less,vpt", [(0, 16), (1, 8)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_few_rows_of_many_tiles(less, vpt, mode):
+    # five tiles of 16 values an SM
+    n, rows = 5 * 4096 * torch.cuda.get_device_properties(0).multi_processor_count - less, 15
+    g = rng.Generator(n, 81, output_mode=mode)
+    got = g.generate_checksum(rows)
+    assert g.last_checksum()["values_per_thread"] == vpt
+    g.close()
+    _same(got, n, 81, rows, output_mode=mode)
+
+
 def test_no_checksum_launch_yet():
     g = rng.Generator(100, 1)
     with pytest.raises(rng.RngError):
