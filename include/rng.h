@@ -287,7 +287,10 @@ int rng_generate_host_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xo
  * iteration, the XOR (row_xor_dev[it-p]) and the wrapping sum modulo 2^64
  * (row_sum_dev[it-p]) of that iteration's values over all streams.  Both
  * arrays are caller-owned device memory of `iterations` uint64 words; the
- * call clears them first.  Ordered on the compute stream. */
+ * call clears them first.  A launch whose rows are split over blocks (as
+ * rng_generate's of few streams) takes a second state array of 8 bytes per
+ * stream when the states are in memory, kept until rng_destroy; where that
+ * cannot be had the launch runs unsplit.  Ordered on the compute stream. */
 int rng_generate_checksum(rng_gen *g, uint64_t iterations, uint64_t *row_xor_dev,
                           uint64_t *row_sum_dev, rng_err **err);
 
